@@ -21,6 +21,7 @@
 #include "../../include/stdd.h"
 #include "common.cuh"
 #include "kernels.h"
+#include "mf_fixed.cuh"
 #include "symbolic.h"
 
 using stdd::FrontDev;
@@ -218,6 +219,8 @@ struct stdd_ctx {
   int fp64_tc = 1;
   bool oz_active() const { return fp64_tc && sym_active() && prec == STDD_PREC_FP64; }
   DBuf d_lsx, d_lsy;
+  DBuf d_sweep;     // the complex128 substitutions' front records
+  DBuf d_fexp;      // exponents of the fixed-point complex128 factors
   DBuf d_segpart;   // partial sums of the grid-split substitution products
   int forced_split = 0;   // STDD_OPT_SWEEP_SPLIT: 0 tuned, else 1, 2, 4, 8 or MF_SPLIT_GRID
   int64_t nfronts = 0, factor_entries = 0;
@@ -617,6 +620,9 @@ MfArgs stdd_ctx::mf_args(int par, bool solve) const {
   a.panel = pivoting ? d_panel.p : nullptr;
   a.sym = sym_active() ? 1 : 0;
   a.segpart = d_segpart.p;
+  a.fexp = d_fexp.as<short>();
+  a.sweep = d_sweep.as<stdd::SweepFront>();
+  a.fx_scale = std::max(-200, std::min(200, (int)std::ilogb(2.0 / (dx * dx) + 2.0 / (dy * dy))));
   a.fp64_tc = oz_active() ? 1 : 0;
   a.lsx = a.sym ? d_lsx.as<double2>() : nullptr;
   a.lsy = a.sym ? d_lsy.as<double2>() : nullptr;
@@ -704,7 +710,7 @@ void stdd_ctx::factor() {
           sp = 8;
         }
         if (sp > 256 / rows) sp = 256 / rows;
-        if (sp > 1 && (cols + stdd::MF_SEG - 1) / stdd::MF_SEG > stdd::MF_MAXSEG) sp = 1;
+        if (!stdd::mf_split_fits(elem() / 2, sp, cols)) sp = 1;
         return sp;
       };
       li.split_up = li.split_up1 = pick(li.rows_up, li.max_p);
@@ -732,9 +738,9 @@ void stdd_ctx::build_strip_levels() {
       l.rows_down = li.rows_down;
       // (the persistent kernel splits within a block only; any split gives
       // the same sums)
-      auto inblock = [](int sp, int cols) {
+      auto inblock = [&](int sp, int cols) {
         if (sp > 8) sp = 8;
-        return (sp > 1 && (cols + stdd::MF_SEG - 1) / stdd::MF_SEG > stdd::MF_MAXSEG) ? 1 : sp;
+        return stdd::mf_split_fits(elem() / 2, sp, cols) ? sp : 1;
       };
       l.split_up = inblock(li.split_up1, li.max_p);
       l.split_down = inblock(li.split_down1, li.max_n);
@@ -837,7 +843,7 @@ void stdd_ctx::build_structure() {
   lvl_up.assign(depth, std::vector<int>(nsub + 1, 0));
   lvl_down.assign(depth, std::vector<int>(nsub + 1, 0));
   int64_t ws_need[2] = {0, 0};
-  int64_t piv_run = 0;
+  int64_t piv_run = 0, exp_run = 0;
   panel_need = 0;
   ub_elems[0] = ub_elems[1] = 0;
   for (int L = 0; L < depth; ++L) {
@@ -869,7 +875,9 @@ void stdd_ctx::build_structure() {
         d.u_off = u_run;
         d.piv_off = piv_run;
         d.pan_off = pan_run;
+        d.exp_off = exp_run;
         piv_run += sf.p;
+        exp_run += stdd::fx_exps(sf.p, sf.b);
         if (sf.p + sf.b > stdd::MF_SMALL) pan_run += (int64_t)sf.p * stdd::MF_NB;
         s_run += (int64_t)sf.b * sf.b;
         u_run += sf.b;
@@ -950,10 +958,10 @@ void stdd_ctx::build_structure() {
   // least one per front: chunk 0 also stores w_p) and of the pivots coming
   // down.  Levels whose row counts fit in 16 use 16-lane row groups (two
   // fronts per warp); wide fronts split their columns over up to 8 row groups.
-  auto pow2_split = [](int cols, int rows) {
+  auto pow2_split = [&](int cols, int rows) {
     int want = (cols + 4 * rows - 1) / (4 * rows), s = 1;
     while (s < want && s < 8) s *= 2;
-    if ((cols + stdd::MF_SEG - 1) / stdd::MF_SEG > stdd::MF_MAXSEG) s = 1;
+    if (!stdd::mf_split_fits(elem() / 2, s, cols)) s = 1;
     return s;
   };
   std::vector<int2> items;
@@ -1014,6 +1022,38 @@ void stdd_ctx::build_structure() {
   upload(d_items, items, stream);
   const size_t E = elem();
   d_fac.alloc(std::max<int64_t>(1, factor_entries) * E);
+  if (prec == STDD_PREC_FP64) {
+    d_fexp.alloc((size_t)std::max<int64_t>(1, exp_run) * sizeof(short));
+    std::vector<stdd::SweepFront> sw(fr.size());
+    for (size_t f = 0; f < fr.size(); ++f) {
+      const FrontDev &d = fr[f];
+      const StripDev &s = sdev[d.strip];
+      stdd::SweepFront &w = sw[f];
+      const int n = d.p + d.b;
+      w.down = d.fac_off;
+      w.up = d.fac_off + (int64_t)d.p * n;
+      w.edown = d.exp_off;
+      w.eup = d.exp_off + stdd::fx_exps_down(d.p, d.b);
+      w.nodes = d.node_off;
+      w.piv = d.piv_off;
+      w.voff = s.vec_off;
+      w.u = d.u_off;
+      w.p = d.p;
+      w.b = d.b;
+      w.Hl = s.y1 - s.y0;
+      w.coef = (int)s.coef_off;
+      w.ycoef = (int)s.ycoef_off;
+      w.pad = 0;
+      for (int ci = 0; ci < 2; ++ci) {
+        const bool has = d.child[ci] >= 0;
+        w.inv[ci] = has ? d.inv_off[ci] : 0;
+        w.uc[ci] = has ? fr[d.child[ci]].u_off : -1;
+        w.bc[ci] = has ? fr[d.child[ci]].b : 0;
+      }
+    }
+    upload(d_sweep, sw, stream);
+    CK(cudaStreamSynchronize(stream));   // sw is on the host's heap
+  }
   d_ws[0].alloc(std::max<int64_t>(1, ws_need[0]) * E);
   d_ws[1].alloc(std::max<int64_t>(1, ws_need[1]) * E);
   solve_nrhs_cap = 0;
@@ -1078,7 +1118,10 @@ template <typename R> void stdd_ctx::autotune() {
               if (rows != 32 || cols <= stdd::MF_SEG) break;
             } else {
               if (sp > 256 / rows) continue;
-              if (sp > 1 && (cols + stdd::MF_SEG - 1) / stdd::MF_SEG > stdd::MF_MAXSEG) continue;
+              if (!stdd::mf_split_fits(sizeof(R), sp, cols)) continue;
+              // more sharers than shares leave warps without work
+              const int share = sizeof(R) == 8 ? stdd::MF_SUB : stdd::MF_SEG;
+              if (sp > 1 && (sp / 2) * share >= cols) continue;
             }
             float ms_min = 1e30f;
             for (int rep = 0; rep < 3; ++rep) {
@@ -1985,7 +2028,7 @@ int64_t stdd_ctx::device_bytes() const {
                        &d_inv, &d_lcxm, &d_lcxp, &d_colstrip, &d_lcym, &d_lcyp, &d_rowbox, &d_fac, &d_ws[0], &d_ws[1], &d_ub[0],
                        &d_ub[1], &d_tloc, &d_wloc, &d_items, &d_flag, &d_minpiv, &d_b, &d_x, &d_r, &d_V, &d_Z, &d_w,
                        &d_part, &d_h, &d_nrm, &d_y, &d_pre, &d_fpart, &d_guess, &d_gscr, &d_pcol, &d_panel,
-                       &d_striplv, &d_bar, &d_sweep_flag, &d_lsx, &d_lsy, &d_segpart};
+                       &d_striplv, &d_bar, &d_sweep_flag, &d_lsx, &d_lsy, &d_segpart, &d_fexp, &d_sweep};
   int64_t s = 0;
   for (auto *d : all) s += (int64_t)d->bytes;
   return s;

@@ -19,6 +19,14 @@ constexpr int MF_MAXSEG = 16;         // segments an item may have when its colu
 constexpr int MF_SPLIT_GRID = 16;     // split value: one warp per (item, sub-segment) anywhere in the grid
 constexpr int MF_SUB = 32;            // columns per chain inside a segment (segment = chains added in order)
 static_assert(MF_SEG % MF_SUB == 0, "segments are whole sub-segments");
+constexpr int MF_MAXCHAIN = 64;       // complex128: chains a block's items may have in all when split
+// whether items of `cols` columns may share them among `split` row groups (complex64: whole segments) or
+// warps (complex128: whole chains) of a block; real: bytes of a real number
+inline bool mf_split_fits(size_t real, int split, int cols) {
+  if (split <= 1) return true;
+  return real == 8 ? (cols + MF_SUB - 1) / MF_SUB <= MF_MAXCHAIN * split / 8
+                   : (cols + MF_SEG - 1) / MF_SEG <= MF_MAXSEG;
+}
 
 // Everything a multifrontal kernel needs (device pointers).
 struct MfArgs {
@@ -61,6 +69,9 @@ struct MfArgs {
   // one partial sum per (work item, column segment, row), summed in segment
   // order by a second launch
   void *segpart;
+  short *fexp;                // complex128: exponents of the fixed-point factors
+  const SweepFront *sweep;    // complex128: one record per front
+  int fx_scale;               // and the power of two Finv's columns are scaled by
 };
 
 struct LevelInfo {

@@ -44,6 +44,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "mf_fixed.cuh"
 
 namespace stdd {
 
@@ -905,14 +906,13 @@ template <int W, typename C> __device__ __forceinline__ C shfl_w(unsigned mask, 
 // acc[q] = sum over columns [c0, c1) of M(r, c) * vec_q(c), q < NR, for one
 // segment; M(r, c) at M[c * ld + r]; vec_q(c) comes from gather(c, q).
 // Each matrix entry is loaded once for all NR right-hand sides.
-template <int ROWS, int NR, bool AHEAD, typename C, typename Gather>
+template <int ROWS, int NR, typename C, typename Gather>
 __device__ __forceinline__ void seg_dot(const C *__restrict__ M, int64_t ld, int r, bool row, int c0, int c1,
                                         int lane, unsigned mask, Gather gather, C (&acc)[NR]) {
   // the next chunk's vector values are requested before this chunk's
   // products (at the top tree levels a few warps carry a whole phase and
   // would otherwise wait for the dependent gather once per chunk)
-  constexpr int U0 = sizeof(C) == 16 ? 8 : 32;  // FP64 is ALU-bound: fewer loads, more warps
-  constexpr int U = NR > 1 ? (U0 / NR > 4 ? U0 / NR : 4) : U0;
+  constexpr int U = NR > 1 ? (32 / NR > 4 ? 32 / NR : 4) : 32;
   constexpr int UU = U < ROWS ? U : ROWS;
   static_assert(MF_SUB % ROWS == 0, "a sub-segment is a whole number of chunks");
   // each MF_SUB columns form a chain of their own (sub), folded into the
@@ -923,17 +923,7 @@ __device__ __forceinline__ void seg_dot(const C *__restrict__ M, int64_t ld, int
   C vn[NR];
 #pragma unroll
   for (int q = 0; q < NR; ++q) vn[q] = c0 + lane < c1 ? gather(c0 + lane, q) : czero<C>();
-  // complex128, one right-hand side, AHEAD (the per-level kernels; the
-  // persistent sweep has no registers to spare): matrix loads run one block of UU
-  // columns ahead of the products (the block after a chunk's last one is
-  // the next chunk's first); complex64 and several right-hand sides keep
-  // one block in registers
-  constexpr bool PIPE = AHEAD && sizeof(C) == 16 && NR == 1;
   C m[UU];
-  if (PIPE && c1 - c0 >= ROWS) {
-#pragma unroll
-    for (int u = 0; u < UU; ++u) m[u] = row ? M[(int64_t)(c0 + u) * ld + r] : czero<C>();
-  }
   for (int cb = c0; cb < c1; cb += ROWS) {
     if ((cb - c0) % MF_SUB == 0) {
 #pragma unroll
@@ -947,29 +937,14 @@ __device__ __forceinline__ void seg_dot(const C *__restrict__ M, int64_t ld, int
     for (int q = 0; q < NR; ++q) vn[q] = cn < c1 ? gather(cn, q) : czero<C>();
     const int nv = min(ROWS, c1 - cb);
     if (nv == ROWS) {
-      const bool next_full = c1 - (cb + ROWS) >= ROWS;
 #pragma unroll
       for (int u0 = 0; u0 < ROWS; u0 += UU) {
-        if (PIPE) {
-          C mn[UU];
-          const int nb = u0 + UU < ROWS ? cb + u0 + UU : cb + ROWS;   // the block loaded ahead
-          const bool ahead = u0 + UU < ROWS || next_full;
 #pragma unroll
-          for (int u = 0; u < UU; ++u) mn[u] = (row && ahead) ? M[(int64_t)(nb + u) * ld + r] : czero<C>();
+        for (int u = 0; u < UU; ++u) m[u] = row ? M[(int64_t)(cb + u0 + u) * ld + r] : czero<C>();
 #pragma unroll
-          for (int u = 0; u < UU; ++u)
+        for (int u = 0; u < UU; ++u)
 #pragma unroll
-            for (int q = 0; q < NR; ++q) sub[q] = cfma(m[u], shfl_w<ROWS>(mask, v[q], u0 + u), sub[q]);
-#pragma unroll
-          for (int u = 0; u < UU; ++u) m[u] = mn[u];
-        } else {
-#pragma unroll
-          for (int u = 0; u < UU; ++u) m[u] = row ? M[(int64_t)(cb + u0 + u) * ld + r] : czero<C>();
-#pragma unroll
-          for (int u = 0; u < UU; ++u)
-#pragma unroll
-            for (int q = 0; q < NR; ++q) sub[q] = cfma(m[u], shfl_w<ROWS>(mask, v[q], u0 + u), sub[q]);
-        }
+          for (int q = 0; q < NR; ++q) sub[q] = cfma(m[u], shfl_w<ROWS>(mask, v[q], u0 + u), sub[q]);
       }
     } else {
       // ragged last chunk: only the valid columns (no multiply-adds by zero)
@@ -996,6 +971,110 @@ __device__ __forceinline__ void seg_dot(const C *__restrict__ M, int64_t ld, int
     }
   }
 }
+
+// Chains [k0, k1) of a complex128 front's block through the fixed-point
+// products (mf_fixed.cuh): one warp, MT x 16 rows from r0, the walk f started
+// at chain k0 and ending with chain k1 - 1.  gather(column, q) is the vector value, expo(column) the power
+// of two its column was scaled by; sink(chain, sums) receives each chain's
+// sums, sums[q][t] the lane's component (lane % 2) of its row (fx_row) of tile t.
+template <int MT, int NR, typename Gather, typename Expo, typename Sink>
+__device__ __forceinline__ void fx_chains(FxRows<MT> &f, int r0, int k0, int k1, int lane, const FxLane &fl,
+                                          ulonglong2 (*xs)[FX_COLS], Gather gather, Expo expo, Sink sink) {
+  const int cend = f.cend;
+  double2 vn[NR];
+  const int cf = k0 * FX_COLS + lane;
+#pragma unroll
+  for (int q = 0; q < NR; ++q) vn[q] = cf < cend ? gather(cf, q) : czero<double2>();
+  for (int k = k0; k < k1; ++k) {
+    const int c0 = k * FX_COLS, col = c0 + lane;
+    const int sh = expo(col);
+    int ex[NR];
+    __syncwarp();      // the previous chain's products have read xs
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+      ex[q] = __reduce_max_sync(0xffffffffu, max(fx_exp(vn[q].x, -sh), fx_exp(vn[q].y, -sh)));
+      xs[q][lane] = make_ulonglong2(fx_vector_word(vn[q].x, ex[q] + sh), fx_vector_word(vn[q].y, ex[q] + sh));
+    }
+    __syncwarp();
+    // the next chain's vector values are requested before this one's products
+    const int cn = col + FX_COLS;
+#pragma unroll
+    for (int q = 0; q < NR; ++q) vn[q] = cn < cend ? gather(cn, q) : czero<double2>();
+    double s[NR][MT];
+    if (f.rows > 0) {
+      fx_chain<MT, NR>(f, r0, c0, lane, fl, xs, ex, s);
+    } else {
+#pragma unroll
+      for (int q = 0; q < NR; ++q)
+#pragma unroll
+        for (int t = 0; t < MT; ++t) s[q][t] = 0.0;
+    }
+    sink(k, s);
+  }
+}
+// row of a 16-row tile whose sum a lane of fx_chain holds
+__device__ __forceinline__ int fx_row(int lane) { return 8 * ((lane >> 1) & 1) + (lane >> 2); }
+// component lane % 2 of v
+__device__ __forceinline__ double fx_part(double2 v, int lane) { return (lane & 1) ? v.y : v.x; }
+
+// Factor blocks of a level's eliminated fronts to fixed point, in place: one
+// warp per 32 rows of a chain, lane = row, 32 columns in registers.  Reads
+// and writes every entry once (a pass at HBM speed; the preconditioner's
+// products then never convert).
+__global__ void __launch_bounds__(128) mf_to_fixed(MfArgs a, int f0, int nf, int upf) {
+  const int64_t w = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  const int fi = (int)(w / upf);
+  int u = (int)(w - (int64_t)fi * upf);
+  if (fi >= nf) return;
+  const FrontDev f = a.fronts[f0 + fi];
+  const int p = f.p, b = f.b, n = p + b;
+  const int nd = (n + FX_COLS - 1) / FX_COLS, nu = (p + FX_COLS - 1) / FX_COLS;
+  const int rd = (p + 31) / 32, ru = (b + 31) / 32;
+  int rows = p, cols = n;
+  int64_t base = f.fac_off, eo = f.exp_off;
+  const bool down = u < rd * nd;
+  if (!down) {
+    u -= rd * nd;
+    if (u >= ru * nu) return;
+    rows = b;
+    cols = p;
+    base += (int64_t)p * n;
+    eo += (int64_t)p * nd;
+  }
+  const int rc = (rows + 31) / 32, ch = u / rc, r = (u - ch * rc) * 32 + lane;
+  if (r >= rows) return;
+  const int c0 = ch * FX_COLS, nc = min(FX_COLS, cols - c0);
+  double2 *M = reinterpret_cast<double2 *>(a.fac) + base + (int64_t)c0 * rows + r;
+  double2 v[FX_COLS];
+  int e = FX_EMPTY;
+  const int scaled = down ? p : 0;      // columns of Finv carry 2^fx_scale
+#pragma unroll
+  for (int k = 0; k < FX_COLS; ++k)
+    if (k < nc) v[k] = M[(int64_t)k * rows];
+#pragma unroll
+  for (int k = 0; k < FX_COLS; ++k)
+    if (k < nc) {
+      const int sh = c0 + k < scaled ? a.fx_scale : 0;
+      e = max(e, max(fx_exp(v[k].x, sh), fx_exp(v[k].y, sh)));
+    }
+  a.fexp[eo + (int64_t)ch * rows + r] = (short)e;
+#pragma unroll
+  for (int k = 0; k < FX_COLS; ++k)
+    if (k < nc) {
+      const int ek = e - (c0 + k < scaled ? a.fx_scale : 0);
+      reinterpret_cast<ulonglong2 *>(M)[(int64_t)k * rows] =
+          make_ulonglong2(fx_matrix_word(v[k].x, ek), fx_matrix_word(v[k].y, ek));
+    }
+}
+
+// The sweeps' launches of consecutive levels overlap (programmatic dependent
+// launch): a block starts while the previous level's last ones still run,
+// loads what the factorization left (items, records, the first matrix
+// entries) and waits for that level's vectors here.  Without the launch
+// attribute both are no-ops.
+__device__ __forceinline__ void level_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void level_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 // Going up, part 1: one warp per front forms w = [t at the pivots; 0] plus
 // the children's update vectors (inverse extend-add maps); w_p goes to the
@@ -1038,6 +1117,23 @@ __device__ __forceinline__ WSrc<C> wsrc_make(const MfArgs &a, const FrontDev &f,
   }
   return w;
 }
+// the same from a complex128 front's record
+__device__ __forceinline__ WSrc<double2> wsrc_make(const MfArgs &a, const SweepFront &f, int nrhs) {
+  WSrc<double2> w;
+  w.nodes = a.nodes + f.nodes;
+  w.voff = f.voff;
+  w.coef_off = f.coef;
+  w.ycoef_off = f.ycoef;
+  w.Hl = f.Hl;
+  w.sym = a.sym != 0;
+#pragma unroll
+  for (int ci = 0; ci < 2; ++ci) {
+    w.inv[ci] = a.inv + f.inv[ci];
+    w.uc[ci] = f.uc[ci] >= 0 ? reinterpret_cast<const double2 *>(a.ub_child) + f.uc[ci] * nrhs : nullptr;
+    w.bc[ci] = f.bc[ci];
+  }
+  return w;
+}
 // children's update vectors at position k, added to w in child order
 template <typename C>
 __device__ __forceinline__ C wsrc_children(const WSrc<C> &s, int k, int q, C w) {
@@ -1057,7 +1153,9 @@ __device__ __forceinline__ C wsrc_pivot(const MfArgs &a, const WSrc<C> &s, int k
   C w = reinterpret_cast<const C *>(a.tloc)[*gi];
   if (s.sym) {   // the source of D A x = D t
     const int ux = node / s.Hl, uy = node - ux * s.Hl;
-    w = cmul(w, to_c(cmul(a.lsx[s.coef_off + ux], a.lsy[s.ycoef_off + uy]), C()));
+    const double2 sx = a.lsx[s.coef_off + ux], sy = a.lsy[s.ycoef_off + uy];
+    // outside the PMLs both stretches are exactly 1
+    if (sx.y != 0.0 || sy.y != 0.0) w = cmul(w, to_c(cmul(sx, sy), C()));
   }
   return wsrc_children(s, k, q, w);
 }
@@ -1102,7 +1200,7 @@ __global__ void __launch_bounds__(256) mf_up_gather(MfArgs a, int f0, int nf, in
 // themselves (WSrc, the gather's own arithmetic), the front's first row
 // chunk stores w_p for the way down, and each row starts from the
 // children's update vectors.
-template <typename R, int ROWS, int NR, bool AHEAD = true, bool FUSED = false>
+template <typename R, int ROWS, int NR, bool FUSED = false>
 __device__ __forceinline__ void up_block(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                          int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
   using C = typename CT<R>::T;
@@ -1162,7 +1260,7 @@ __device__ __forceinline__ void up_block(const MfArgs &a, const int2 *__restrict
       };
       for (int sg = seg0; sg < seg1; ++sg) {
         C sv[NR];
-        seg_dot<ROWS, NR, AHEAD, C>(G, b, r, row, sg * MF_SEG, min(p, (sg + 1) * MF_SEG), lane, mask, gather, sv);
+        seg_dot<ROWS, NR, C>(G, b, r, row, sg * MF_SEG, min(p, (sg + 1) * MF_SEG), lane, mask, gather, sv);
         if (split == 1) {
 #pragma unroll
           for (int q = 0; q < NR; ++q) total[q] = cadd(total[q], sv[q]);
@@ -1189,7 +1287,7 @@ __device__ __forceinline__ void up_block(const MfArgs &a, const int2 *__restrict
 // Coming down: lane = pivot row r;
 // x[r] = sum_{c<p} Finv(r, c) w_p[c] - sum_{c>=p} H12(r, c) x_b[c].
 // one (virtual) block of the downward products: the items of block vb
-template <typename R, int ROWS, int NR, bool AHEAD = true>
+template <typename R, int ROWS, int NR>
 __device__ __forceinline__ void down_block(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                            int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
   using C = typename CT<R>::T;
@@ -1234,7 +1332,7 @@ __device__ __forceinline__ void down_block(const MfArgs &a, const int2 *__restri
       };
       for (int sg = seg0; sg < seg1; ++sg) {
         C sv[NR];
-        seg_dot<ROWS, NR, AHEAD, C>(Fm, p, r, row, sg * MF_SEG, min(n, (sg + 1) * MF_SEG), lane, mask, gather, sv);
+        seg_dot<ROWS, NR, C>(Fm, p, r, row, sg * MF_SEG, min(n, (sg + 1) * MF_SEG), lane, mask, gather, sv);
         if (split == 1) {
 #pragma unroll
           for (int q = 0; q < NR; ++q) total[q] = cadd(total[q], sv[q]);
@@ -1258,19 +1356,245 @@ __device__ __forceinline__ void down_block(const MfArgs &a, const int2 *__restri
   }
 }
 
+// The same two blocks for complex128 fronts, whose factors are fixed-point
+// numbers: one warp per work item (MT x 16 rows) or per share of its chains.
+// Chain sums are folded as in complex64: four to a segment sum, the segment
+// sums added in column order, so the split changes no result.  With split > 1
+// the chain sums meet in `part`, which holds MF_MAXCHAIN chains of 32 rows.
+// `total` of each row plus its segment sums, chain by chain in column order
+template <int MT, int NR> struct FxFold {
+  double total[NR][MT], seg[NR][MT];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int q = 0; q < NR; ++q)
+#pragma unroll
+      for (int t = 0; t < MT; ++t) total[q][t] = seg[q][t] = 0.0;
+  }
+  __device__ __forceinline__ void add(int q, int t, int k, int nk, double s) {
+    constexpr int PER = MF_SEG / FX_COLS;
+    seg[q][t] = k % PER == 0 ? s : seg[q][t] + s;
+    if (k % PER == PER - 1 || k == nk - 1) total[q][t] += seg[q][t];
+  }
+};
+
+template <int MT, int NR, bool FUSED, bool PDL>
+__device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
+                                            int nrhs, int64_t ldt, int vb, double *part,
+                                            ulonglong2 (*xs)[FX_COLS]) {
+  const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ipc = 8 / split, il = g / split, sidx = g - il * split;
+  const int it = vb * ipc + il;
+  const bool active = it < nitems;
+  const FxLane fl(lane);
+  int p = 0, b = 0, r0 = 0, k0 = 0, k1 = 0, nk = 0;
+  const double2 *G = nullptr;
+  const short *E = nullptr;
+  const int *nodes = nullptr, *pc = nullptr;
+  int64_t voff = 0;
+  double2 *u = nullptr;
+  WSrc<double2> src;
+  bool writer = false;
+  if (active) {
+    const int2 item = items[it];
+    const SweepFront f = a.sweep[item.x];
+    p = f.p;
+    b = f.b;
+    voff = f.voff;
+    if (FUSED) {
+      src = wsrc_make(a, f, nrhs);
+      writer = item.y == 0;
+    }
+    G = reinterpret_cast<const double2 *>(a.fac) + f.up;   // -G21, b x p, ld b
+    E = a.fexp + f.eup;
+    r0 = item.y * 16 * MT;
+    nodes = a.nodes + f.nodes;
+    u = reinterpret_cast<double2 *>(a.ub_cur) + f.u * nrhs;
+    if (a.pcol) pc = a.pcol + f.piv;
+    nk = (p + FX_COLS - 1) / FX_COLS;
+    k0 = sidx * nk / split;
+    k1 = (sidx + 1) * nk / split;
+  }
+  double2 *wl = reinterpret_cast<double2 *>(a.wloc);
+  double *mine = part + (int64_t)il * (MF_MAXCHAIN * split / 8) * MT * 32 + lane;
+  for (int q0 = 0; q0 < nrhs; q0 += NR) {
+    FxRows<MT> f;
+    f.start(G, E, r0, b, k0 * FX_COLS, min(p, k1 * FX_COLS), lane);
+    if (PDL) level_wait();
+    double w0[NR][MT];     // the children's update vectors at the item's rows
+#pragma unroll
+    for (int q = 0; q < NR; ++q)
+#pragma unroll
+      for (int t = 0; t < MT; ++t) {
+        const int r = r0 + 16 * t + fx_row(lane);
+        const int64_t at = (int64_t)(q0 + q) * b + r;
+        w0[q][t] = 0.0;
+        if (sidx == 0 && r < b && q0 + q < nrhs)
+          w0[q][t] = fx_part(FUSED ? wsrc_children(src, p + r, q0 + q, czero<double2>()) : u[at], lane);
+      }
+    FxFold<MT, NR> fold;
+    fold.clear();
+    if (k0 < k1) {
+      auto gather = [&](int j, int q) {
+        if (q0 + q >= nrhs) return czero<double2>();
+        if (!FUSED) return wl[(q0 + q) * ldt + voff + nodes[pc ? pc[j] : j]];
+        int64_t gi;
+        const double2 w = wsrc_pivot(a, src, pc ? pc[j] : j, q0 + q, ldt, &gi);
+        if (writer) wl[gi] = w;
+        return w;
+      };
+      fx_chains<MT, NR>(f, r0, k0, k1, lane, fl, xs, gather, [](int) { return 0; },
+                        [&](int k, const double(&s)[NR][MT]) {
+#pragma unroll
+                          for (int t = 0; t < MT; ++t)
+                            if (split == 1) {
+#pragma unroll
+                              for (int q = 0; q < NR; ++q) fold.add(q, t, k, nk, s[q][t]);
+                            } else {
+                              mine[(k * MT + t) * 32] = s[0][t];
+                            }
+                        });
+    }
+    if (split > 1) __syncthreads();
+    if (active && sidx == 0) {
+#pragma unroll
+      for (int t = 0; t < MT; ++t) {
+        const int r = r0 + 16 * t + fx_row(lane);
+        if (split > 1)
+          for (int k = 0; k < nk; ++k) fold.add(0, t, k, nk, mine[(k * MT + t) * 32]);
+        if (r < b)
+#pragma unroll
+          for (int q = 0; q < NR; ++q)
+            if (q0 + q < nrhs)
+              reinterpret_cast<double *>(u)[2 * ((int64_t)(q0 + q) * b + r) + (lane & 1)] = w0[q][t] + fold.total[q][t];
+      }
+    }
+    if (split > 1) __syncthreads();
+  }
+}
+
+template <int MT, int NR, bool PDL>
+__device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
+                                              int nrhs, int64_t ldt, int vb, double *part,
+                                              ulonglong2 (*xs)[FX_COLS]) {
+  const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ipc = 8 / split, il = g / split, sidx = g - il * split;
+  const int it = vb * ipc + il;
+  const bool active = it < nitems;
+  const FxLane fl(lane);
+  int p = 0, n = 0, r0 = 0, k0 = 0, k1 = 0, nk = 0;
+  const double2 *Fm = nullptr;
+  const short *E = nullptr;
+  const int *nodes = nullptr, *pc = nullptr;
+  int64_t voff = 0;
+  if (active) {
+    const int2 item = items[it];
+    const SweepFront f = a.sweep[item.x];
+    p = f.p;
+    n = p + f.b;
+    voff = f.voff;
+    Fm = reinterpret_cast<const double2 *>(a.fac) + f.down;   // p x n, ld p
+    E = a.fexp + f.edown;
+    r0 = item.y * 16 * MT;
+    nodes = a.nodes + f.nodes;
+    if (a.pcol) pc = a.pcol + f.piv;
+    nk = (n + FX_COLS - 1) / FX_COLS;
+    k0 = sidx * nk / split;
+    k1 = (sidx + 1) * nk / split;
+  }
+  double2 *tv = reinterpret_cast<double2 *>(a.tloc);
+  const double2 *wl = reinterpret_cast<const double2 *>(a.wloc);
+  double *mine = part + (int64_t)il * (MF_MAXCHAIN * split / 8) * MT * 32 + lane;
+  for (int q0 = 0; q0 < nrhs; q0 += NR) {
+    FxRows<MT> f;
+    f.start(Fm, E, r0, p, k0 * FX_COLS, min(n, k1 * FX_COLS), lane);
+    if (PDL) level_wait();
+    FxFold<MT, NR> fold;
+    fold.clear();
+    if (k0 < k1) {
+      auto gather = [&](int c, int q) {
+        if (q0 + q >= nrhs) return czero<double2>();
+        const int64_t base = (q0 + q) * ldt + voff;
+        return c < p ? wl[base + nodes[pc ? pc[c] : c]] : cneg(tv[base + nodes[c]]);
+      };
+      fx_chains<MT, NR>(f, r0, k0, k1, lane, fl, xs, gather,
+                        [&](int c) { return c < p ? a.fx_scale : 0; },
+                        [&](int k, const double(&s)[NR][MT]) {
+#pragma unroll
+                          for (int t = 0; t < MT; ++t)
+                            if (split == 1) {
+#pragma unroll
+                              for (int q = 0; q < NR; ++q) fold.add(q, t, k, nk, s[q][t]);
+                            } else {
+                              mine[(k * MT + t) * 32] = s[0][t];
+                            }
+                        });
+    }
+    if (split > 1) __syncthreads();
+    if (active && sidx == 0) {
+#pragma unroll
+      for (int t = 0; t < MT; ++t) {
+        const int r = r0 + 16 * t + fx_row(lane);
+        if (split > 1)
+          for (int k = 0; k < nk; ++k) fold.add(0, t, k, nk, mine[(k * MT + t) * 32]);
+        if (r < p)
+#pragma unroll
+          for (int q = 0; q < NR; ++q)
+            if (q0 + q < nrhs)
+              reinterpret_cast<double *>(tv)[2 * ((q0 + q) * ldt + voff + nodes[r]) + (lane & 1)] = fold.total[q][t];
+      }
+    }
+    if (split > 1) __syncthreads();
+  }
+}
+
+// A work item's rows (16 or 32) go to one warp in complex128, to as many
+// lanes in complex64: items a 256-thread block holds at split 1.
+template <typename R> __host__ __device__ constexpr int block_items(int rows) {
+  return sizeof(R) == 8 ? 8 : 256 / rows;
+}
+
+// one (virtual) block of products of either precision; `part` holds the
+// segment sums of split items, the warps' vector words follow it
+template <typename R, int NR>
+constexpr int SWEEP_SMEM = MF_MAXSEG * 256 / 2 + (sizeof(R) == 8 ? 8 * NR * FX_COLS : 0);
+template <typename R, int ROWS, int NR, bool FUSED, bool PDL>
+__device__ __forceinline__ void up_any(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
+                                       int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
+  if constexpr (sizeof(R) == 8) {
+    auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_MAXSEG * 256 / 2) + (threadIdx.x >> 5) * NR;
+    up_block_fx<ROWS / 16, NR, FUSED, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs);
+  } else {
+    if (PDL) level_wait();
+    up_block<R, ROWS, NR, FUSED>(a, items, nitems, split, nrhs, ldt, vb, part);
+  }
+}
+template <typename R, int ROWS, int NR, bool PDL>
+__device__ __forceinline__ void down_any(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
+                                         int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
+  if constexpr (sizeof(R) == 8) {
+    auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_MAXSEG * 256 / 2) + (threadIdx.x >> 5) * NR;
+    down_block_fx<ROWS / 16, NR, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs);
+  } else {
+    if (PDL) level_wait();
+    down_block<R, ROWS, NR>(a, items, nitems, split, nrhs, ldt, vb, part);
+  }
+}
+
 template <typename R, int ROWS, int NR, bool FUSED>
 __global__ void __launch_bounds__(256, 2) mf_up(MfArgs a, const int2 *__restrict__ items,
                                                                      int nitems, int split, int nrhs, int64_t ldt) {
-  __shared__ typename CT<R>::T part[MF_MAXSEG * 256 / 2];
-  up_block<R, ROWS, NR, true, FUSED>(a, items, nitems, split, nrhs, ldt, blockIdx.x, part);
+  __shared__ typename CT<R>::T part[SWEEP_SMEM<R, NR>];
+  level_go();
+  up_any<R, ROWS, NR, FUSED, true>(a, items, nitems, split, nrhs, ldt, blockIdx.x, part);
 }
 
 template <typename R, int ROWS, int NR>
 __global__ void __launch_bounds__(256, 2) mf_down(MfArgs a, const int2 *__restrict__ items,
                                                                        int nitems, int split, int nrhs,
                                                                        int64_t ldt) {
-  __shared__ typename CT<R>::T part[MF_MAXSEG * 256 / 2];
-  down_block<R, ROWS, NR>(a, items, nitems, split, nrhs, ldt, blockIdx.x, part);
+  __shared__ typename CT<R>::T part[SWEEP_SMEM<R, NR>];
+  level_go();
+  down_any<R, ROWS, NR, true>(a, items, nitems, split, nrhs, ldt, blockIdx.x, part);
 }
 
 // Products split across the grid: one warp per (work item, MF_SUB-column
@@ -1284,6 +1608,7 @@ template <typename R, bool UP, bool FUSED>
 __global__ void __launch_bounds__(256) mf_seg_partial(MfArgs a, const int2 *__restrict__ items, int nitems,
                                                       int nsubmax, int64_t ldt) {
   using C = typename CT<R>::T;
+  level_go();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t u = (int64_t)blockIdx.x * 8 + warp;
   if (u >= (int64_t)nitems * nsubmax) return;
@@ -1301,33 +1626,47 @@ __global__ void __launch_bounds__(256) mf_seg_partial(MfArgs a, const int2 *__re
   const C *fac = reinterpret_cast<const C *>(a.fac) + f.fac_off;
   const int r = item.y * 32 + lane;
   const bool row = r < (UP ? b : p);
-  C sv[1];
-  if (UP) {
-    WSrc<C> src;
-    if (FUSED) src = wsrc_make<C>(a, f, 1);
-    auto gather = [&](int j, int) {
-      if (!FUSED) return wl[voff + nodes[pc ? pc[j] : j]];
-      int64_t gi;
-      const C w = wsrc_pivot(a, src, pc ? pc[j] : j, 0, ldt, &gi);
-      if (item.y == 0) const_cast<C *>(wl)[gi] = w;
-      return w;
-    };
-    seg_dot<32, 1, true, C>(fac + (int64_t)p * n, b, r, row, sg * MF_SUB, min(cols, (sg + 1) * MF_SUB), lane,
-                            0xffffffffu, gather, sv);
+  const int c0 = sg * MF_SUB, c1 = min(cols, c0 + MF_SUB);
+  const C *M = UP ? fac + (int64_t)p * n : fac;
+  const int ld = UP ? b : p;
+  WSrc<C> src;
+  if (UP && FUSED) src = wsrc_make<C>(a, f, 1);
+  auto gather = [&](int j, int) {
+    if (!UP) return j < p ? wl[voff + nodes[pc ? pc[j] : j]] : cneg(tv[voff + nodes[j]]);
+    if (!FUSED) return wl[voff + nodes[pc ? pc[j] : j]];
+    int64_t gi;
+    const C w = wsrc_pivot(a, src, pc ? pc[j] : j, 0, ldt, &gi);
+    if (item.y == 0) const_cast<C *>(wl)[gi] = w;
+    return w;
+  };
+  if constexpr (sizeof(R) == 8) {
+    __shared__ ulonglong2 xs[8][1][FX_COLS];
+    const FxLane fl(lane);
+    const short *E = a.fexp + f.exp_off + (UP ? (int64_t)p * ((n + FX_COLS - 1) / FX_COLS) : 0);
+    double *out = reinterpret_cast<double *>(a.segpart) + u * 64 + 2 * fx_row(lane) + (lane & 1);
+    FxRows<2> walk;
+    walk.start(M, E, item.y * 32, ld, c0, c1, lane);
+    level_wait();
+    fx_chains<2, 1>(walk, item.y * 32, sg, sg + 1, lane, fl, xs[warp], gather,
+                    [&](int c) { return !UP && c < p ? a.fx_scale : 0; },
+                    [&](int, const double(&s)[1][2]) {
+                      out[0] = s[0][0];
+                      out[32] = s[0][1];
+                    });
   } else {
-    auto gather = [&](int c, int) {
-      return c < p ? wl[voff + nodes[pc ? pc[c] : c]] : cneg(tv[voff + nodes[c]]);
-    };
-    seg_dot<32, 1, true, C>(fac, p, r, row, sg * MF_SUB, min(cols, (sg + 1) * MF_SUB), lane, 0xffffffffu, gather,
-                            sv);
+    C sv[1];
+    level_wait();
+    seg_dot<32, 1, C>(M, ld, r, row, c0, c1, lane, 0xffffffffu, gather, sv);
+    reinterpret_cast<C *>(a.segpart)[u * 32 + lane] = sv[0];
   }
-  reinterpret_cast<C *>(a.segpart)[u * 32 + lane] = sv[0];
 }
 
 template <typename R, bool UP, bool FUSED>
 __global__ void __launch_bounds__(256) mf_seg_reduce(MfArgs a, const int2 *__restrict__ items, int nitems,
                                                      int nsubmax) {
   using C = typename CT<R>::T;
+  level_go();
+  level_wait();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int it = (int)(t >> 5), lane = (int)(t & 31);
   if (it >= nitems) return;
@@ -1340,24 +1679,42 @@ __global__ void __launch_bounds__(256) mf_seg_reduce(MfArgs a, const int2 *__res
   const int nsub = (cols + MF_SUB - 1) / MF_SUB, per = MF_SEG / MF_SUB;
   const C *P = reinterpret_cast<const C *>(a.segpart) + (int64_t)it * nsubmax * 32 + lane;
   C *u = reinterpret_cast<C *>(a.ub_cur) + f.u_off;
-  C total = czero<C>();
-  if (UP) total = FUSED ? wsrc_children(wsrc_make<C>(a, f, 1), p + r, 0, czero<C>()) : u[r];
+  C w0 = czero<C>(), total = czero<C>();
+  if (UP) w0 = FUSED ? wsrc_children(wsrc_make<C>(a, f, 1), p + r, 0, czero<C>()) : u[r];
+  if (sizeof(R) == 4) total = w0;      // complex64 items start from it, complex128 ones add it last
   for (int k0 = 0; k0 < nsub; k0 += per) {
     C seg = P[k0 * 32];
     for (int k = k0 + 1; k < min(k0 + per, nsub); ++k) seg = cadd(seg, P[k * 32]);
     total = cadd(total, seg);
   }
+  if (sizeof(R) == 8) total = cadd(w0, total);
   if (UP) u[r] = total;
   else reinterpret_cast<C *>(a.tloc)[a.strips[f.strip].vec_off + a.nodes[f.node_off + r]] = total;
+}
+
+// 256-thread blocks that may start before the stream's previous kernel ends
+// (the kernel calls level_wait before it reads what that one writes)
+template <typename... P, typename... A>
+void launch_overlapped(void (*kernel)(P...), unsigned grid, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);   // errors: cudaGetLastError by the caller
 }
 
 template <typename R, bool UP, bool FUSED = false>
 void mf_seg_launch(const MfArgs &a, const int2 *items, int nitems, int cols_max, int64_t ldt, cudaStream_t st) {
   const int nsubmax = (cols_max + MF_SUB - 1) / MF_SUB;
   const int64_t units = (int64_t)nitems * nsubmax;
-  mf_seg_partial<R, UP, FUSED><<<(unsigned)((units + 7) / 8), 256, 0, st>>>(a, items, nitems, nsubmax, ldt);
-  mf_seg_reduce<R, UP, FUSED><<<(unsigned)(((int64_t)nitems * 32 + 255) / 256), 256, 0, st>>>(a, items, nitems,
-                                                                                              nsubmax);
+  launch_overlapped(mf_seg_partial<R, UP, FUSED>, (unsigned)((units + 7) / 8), st, a, items, nitems, nsubmax, ldt);
+  launch_overlapped(mf_seg_reduce<R, UP, FUSED>, (unsigned)(((int64_t)nitems * 32 + 255) / 256), st, a, items,
+                    nitems, nsubmax);
   count_launch(2);
 }
 
@@ -1399,19 +1756,19 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *flag, long long
 template <typename R, int ROWS>
 __device__ __forceinline__ void up_items(const MfArgs &a, const StripLevel &l, int64_t ldt,
                                          typename CT<R>::T *part) {
-  const int ipc = (256 / ROWS) / l.split_up;
+  const int ipc = block_items<R>(ROWS) / l.split_up;
   const int nvb = (l.up_n + ipc - 1) / ipc;
   for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x)
-    up_block<R, ROWS, 1, false, true>(a, a.items_sweep + l.up_first, l.up_n, l.split_up, 1, ldt, vb, part);
+    up_any<R, ROWS, 1, true, false>(a, a.items_sweep + l.up_first, l.up_n, l.split_up, 1, ldt, vb, part);
 }
 
 template <typename R, int ROWS>
 __device__ __forceinline__ void down_items(const MfArgs &a, const StripLevel &l, int64_t ldt,
                                            typename CT<R>::T *part) {
-  const int ipc = (256 / ROWS) / l.split_down;
+  const int ipc = block_items<R>(ROWS) / l.split_down;
   const int nvb = (l.down_n + ipc - 1) / ipc;
   for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x)
-    down_block<R, ROWS, 1, false>(a, a.items_sweep + l.down_first, l.down_n, l.split_down, 1, ldt, vb, part);
+    down_any<R, ROWS, 1, false>(a, a.items_sweep + l.down_first, l.down_n, l.split_down, 1, ldt, vb, part);
 }
 
 // The launches of one strip's solve in the sequential orders (residual
@@ -1424,7 +1781,7 @@ __global__ void __launch_bounds__(256, 2)
                    int depth, const double2 *__restrict__ v, double2 *__restrict__ z, unsigned *bar, int *flag,
                    long long limit, int64_t ldt) {
   using C = typename CT<R>::T;
-  __shared__ C part[MF_MAXSEG * 256 / 2];
+  __shared__ C part[SWEEP_SMEM<R, 1>];
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int Hl = s.y1 - s.y0;
   const int64_t nl = (int64_t)(s.x1 - s.x0) * Hl;
@@ -1551,6 +1908,13 @@ void mf_factor_level(const MfArgs &a, const LevelInfo &L, int level, cudaStream_
       count_launch(4);
     }
   }
+  if constexpr (sizeof(R) == 8) {
+    // the substitutions read fixed-point factors (the parents only read S)
+    const int upf = (L.max_p + 31) / 32 * ((L.max_n + FX_COLS - 1) / FX_COLS) +
+                    (L.max_b + 31) / 32 * ((L.max_p + FX_COLS - 1) / FX_COLS);
+    mf_to_fixed<<<(unsigned)(((int64_t)L.nf * upf + 3) / 4), 128, 0, st>>>(a, L.f0, L.nf, upf);
+    count_launch();
+  }
 }
 
 template <typename R>
@@ -1574,19 +1938,20 @@ void mf_up_level(const MfArgs &a, const int2 *items, int nitems, int rows, int s
     }
     split = 1;
   }
-  if (split > 1 && cols_max > 0 && (cols_max + MF_SEG - 1) / MF_SEG > MF_MAXSEG) split = 1;
-  const int ipc = (256 / rows) / split;
+  if (cols_max > 0 && !mf_split_fits(sizeof(R), split, cols_max)) split = 1;
+  const int ipc = block_items<R>(rows) / split;
   const int grid = (nitems + ipc - 1) / ipc;
-  const int nr = (nrhs >= 4 && sizeof(R) == 4) ? 4 : (nrhs >= 2 ? 2 : 1);
+  constexpr int MAXR = sizeof(R) == 4 ? 4 : 2;   // right-hand sides per factor read
+  const int nr = (nrhs >= 4 && MAXR == 4) ? 4 : (nrhs >= 2 ? 2 : 1);
 #define STDD_UP(RW, NRV)                                                                \
   do {                                                                                  \
-    if (fused) mf_up<R, RW, NRV, true><<<grid, 256, 0, st>>>(a, items, nitems, split, nrhs, ldt);  \
-    else mf_up<R, RW, NRV, false><<<grid, 256, 0, st>>>(a, items, nitems, split, nrhs, ldt);       \
+    if (fused) launch_overlapped(mf_up<R, RW, NRV, true>, grid, st, a, items, nitems, split, nrhs, ldt);  \
+    else launch_overlapped(mf_up<R, RW, NRV, false>, grid, st, a, items, nitems, split, nrhs, ldt);       \
   } while (0)
   if (rows == 16) {
-    if (nr == 4) STDD_UP(16, 4); else if (nr == 2) STDD_UP(16, 2); else STDD_UP(16, 1);
+    if (nr == 4) STDD_UP(16, MAXR); else if (nr == 2) STDD_UP(16, 2); else STDD_UP(16, 1);
   } else {
-    if (nr == 4) STDD_UP(32, 4); else if (nr == 2) STDD_UP(32, 2); else STDD_UP(32, 1);
+    if (nr == 4) STDD_UP(32, MAXR); else if (nr == 2) STDD_UP(32, 2); else STDD_UP(32, 1);
   }
 #undef STDD_UP
   count_launch();
@@ -1604,15 +1969,16 @@ void mf_down_level(const MfArgs &a, const int2 *items, int nitems, int rows, int
     }
     split = 1;
   }
-  if (split > 1 && cols_max > 0 && (cols_max + MF_SEG - 1) / MF_SEG > MF_MAXSEG) split = 1;
-  const int ipc = (256 / rows) / split;
+  if (cols_max > 0 && !mf_split_fits(sizeof(R), split, cols_max)) split = 1;
+  const int ipc = block_items<R>(rows) / split;
   const int grid = (nitems + ipc - 1) / ipc;
-  const int nr = (nrhs >= 4 && sizeof(R) == 4) ? 4 : (nrhs >= 2 ? 2 : 1);
-#define STDD_DOWN(RW, NRV) mf_down<R, RW, NRV><<<grid, 256, 0, st>>>(a, items, nitems, split, nrhs, ldt)
+  constexpr int MAXR = sizeof(R) == 4 ? 4 : 2;   // right-hand sides per factor read
+  const int nr = (nrhs >= 4 && MAXR == 4) ? 4 : (nrhs >= 2 ? 2 : 1);
+#define STDD_DOWN(RW, NRV) launch_overlapped(mf_down<R, RW, NRV>, grid, st, a, items, nitems, split, nrhs, ldt)
   if (rows == 16) {
-    if (nr == 4) STDD_DOWN(16, 4); else if (nr == 2) STDD_DOWN(16, 2); else STDD_DOWN(16, 1);
+    if (nr == 4) STDD_DOWN(16, MAXR); else if (nr == 2) STDD_DOWN(16, 2); else STDD_DOWN(16, 1);
   } else {
-    if (nr == 4) STDD_DOWN(32, 4); else if (nr == 2) STDD_DOWN(32, 2); else STDD_DOWN(32, 1);
+    if (nr == 4) STDD_DOWN(32, MAXR); else if (nr == 2) STDD_DOWN(32, 2); else STDD_DOWN(32, 1);
   }
 #undef STDD_DOWN
   count_launch();
