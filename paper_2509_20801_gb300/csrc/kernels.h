@@ -188,6 +188,10 @@ __device__ __forceinline__ double2 grid_row(const GridDev &g, const double2 *__r
 void launch_stencil(const GridDev &g, const double2 *x, double2 *y, cudaStream_t st);
 // r = b - A x
 void launch_residual(const GridDev &g, const double2 *b, const double2 *x, double2 *r, cudaStream_t st);
+// the same (r may be b, not x) with norms2 = (||r||^2, ||b||^2); partial: residual_norm_partials(g) pairs
+void launch_residual_norm(const GridDev &g, const double2 *b, const double2 *x, double2 *r, double2 *partial,
+                          double2 *norms2, cudaStream_t st);
+int64_t residual_norm_partials(const GridDev &g);
 // local[k] = R_k^I v (owned columns of v, zero elsewhere), all strips, R = double or float
 template <typename R>
 void launch_restrict(const StripDev *strips_dev, int nsub, int64_t nloc, int ny, const int *col_strip,

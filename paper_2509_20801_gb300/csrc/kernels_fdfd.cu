@@ -34,33 +34,103 @@ __device__ __forceinline__ double2 apply_row(const GridDev &g, const double2 *__
   return apply_row_ij(g, x, idx, i, j);
 }
 
-// grid-stride walk over all nodes with (i, j) advanced incrementally (no
-// division per node): f(idx, i, j) for every node of this thread
-template <typename F> __device__ __forceinline__ void for_nodes(const GridDev &g, F f) {
-  const int64_t n = (int64_t)g.nx * g.ny, stride = (int64_t)gridDim.x * TPB;
-  int64_t idx = (int64_t)blockIdx.x * TPB + threadIdx.x;
-  if (idx >= n) return;
-  int i = (int)(idx / g.ny), j = (int)(idx - (int64_t)i * g.ny);
-  const int si = (int)(stride / g.ny), sj = (int)(stride - (int64_t)si * g.ny);
-  for (; idx < n; idx += stride) {
-    f(idx, i, j);
-    i += si;
-    j += sj;
-    if (j >= g.ny) {
-      j -= g.ny;
-      ++i;
+// y = A x, or y = b - A x (RES), column by column: a thread keeps its row j
+// and walks ci columns, so the x-neighbours are the values it just had and
+// its y couplings stay in registers.  What bounds it is the FP64 pipe (1 flop
+// a byte against the machine's 0.16): 12 operations a node outside the PML,
+// where the couplings are real, against 15 when every node recomputes the sum
+// of its four couplings, and one new field value a node against three.  b may
+// be y itself (a node is read before it is written, by the same thread).
+// NORM: partial[block] = (sum |y|^2, sum |b|^2) of the block's nodes.
+constexpr int COLT = 128;
+
+template <bool RES, bool NORM>
+__global__ void __launch_bounds__(COLT) k_stencil_cols(GridDev g, const double2 *__restrict__ x, const double2 *b,
+                                                       double2 *y, int ci, double2 *__restrict__ partial) {
+  const int j = blockIdx.x * COLT + threadIdx.x;
+  const int i0 = blockIdx.y * ci, i1 = min(g.nx, i0 + ci);
+  double ny2 = 0.0, nb2 = 0.0;
+  if (j < g.ny) {
+    const double2 ym = g.cym[j], yp = g.cyp[j], zero = make_double2(0.0, 0.0);
+    const bool yreal = ym.y == 0.0 && yp.y == 0.0;
+    const double ys = ym.x + yp.x;
+    const bool has_s = j > 0, has_n = j < g.ny - 1;
+    int64_t idx = (int64_t)i0 * g.ny + j;
+    double2 w = i0 > 0 ? x[idx - g.ny] : zero, c = x[idx];
+    for (int i = i0; i < i1; ++i, idx += g.ny) {
+      const double2 e = i < g.nx - 1 ? x[idx + g.ny] : zero;
+      const double2 s = has_s ? x[idx - 1] : zero, n = has_n ? x[idx + 1] : zero;
+      const double2 xm = g.cxm[i], xp = g.cxp[i];
+      const double2 bv = RES ? b[idx] : zero;
+      const double ke = g.eps[idx];
+      double2 acc;
+      if (yreal && xm.y == 0.0 && xp.y == 0.0) {
+        const double sg = RES ? -1.0 : 1.0;
+        const double d = sg * (fma(g.k0sq, ke, -ys) - (xm.x + xp.x));
+        acc.x = fma(d, c.x, bv.x);
+        acc.y = fma(d, c.y, bv.y);
+        acc.x = fma(sg * xm.x, w.x, acc.x);
+        acc.y = fma(sg * xm.x, w.y, acc.y);
+        acc.x = fma(sg * xp.x, e.x, acc.x);
+        acc.y = fma(sg * xp.x, e.y, acc.y);
+        acc.x = fma(sg * ym.x, s.x, acc.x);
+        acc.y = fma(sg * ym.x, s.y, acc.y);
+        acc.x = fma(sg * yp.x, n.x, acc.x);
+        acc.y = fma(sg * yp.x, n.y, acc.y);
+      } else {
+        const double2 d = make_double2(fma(g.k0sq, ke, -ys) - (xm.x + xp.x), -(xm.y + xp.y) - (ym.y + yp.y));
+        acc = cfma(xm, w, cmul(d, c));
+        acc = cfma(xp, e, acc);
+        acc = cfma(ym, s, acc);
+        acc = cfma(yp, n, acc);
+        if (RES) acc = csub(bv, acc);
+      }
+      y[idx] = acc;
+      if (NORM) {
+        ny2 = fma(acc.x, acc.x, fma(acc.y, acc.y, ny2));
+        nb2 = fma(bv.x, bv.x, fma(bv.y, bv.y, nb2));
+      }
+      w = c;
+      c = e;
+    }
+  }
+  if (NORM) {
+    __shared__ double2 sh[COLT / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      ny2 += __shfl_xor_sync(0xffffffffu, ny2, o);
+      nb2 += __shfl_xor_sync(0xffffffffu, nb2, o);
+    }
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = make_double2(ny2, nb2);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double2 t = sh[0];
+      for (int k = 1; k < COLT / 32; ++k) t = cadd(t, sh[k]);
+      partial[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = t;
     }
   }
 }
 
-__global__ void __launch_bounds__(TPB) k_stencil(GridDev g, const double2 *__restrict__ x, double2 *__restrict__ y) {
-  for_nodes(g, [&](int64_t idx, int i, int j) { y[idx] = apply_row_ij(g, x, idx, i, j); });
+// out = the partial pairs added in a fixed order (one block)
+__global__ void __launch_bounds__(TPB) k_sum_pairs(const double2 *__restrict__ partial, int64_t n,
+                                                   double2 *__restrict__ out) {
+  __shared__ double2 sh[TPB];
+  double2 t = make_double2(0.0, 0.0);
+  for (int64_t k = threadIdx.x; k < n; k += TPB) t = cadd(t, partial[k]);
+  sh[threadIdx.x] = t;
+  for (int o = TPB / 2; o > 0; o >>= 1) {
+    __syncthreads();
+    if (threadIdx.x < o) sh[threadIdx.x] = cadd(sh[threadIdx.x], sh[threadIdx.x + o]);
+  }
+  if (threadIdx.x == 0) out[0] = sh[0];
 }
 
-__global__ void __launch_bounds__(TPB) k_residual(GridDev g, const double2 *__restrict__ b,
-                                                  const double2 *__restrict__ x, double2 *__restrict__ r) {
-  for_nodes(g, [&](int64_t idx, int i, int j) { r[idx] = csub(b[idx], apply_row_ij(g, x, idx, i, j)); });
+// columns a thread walks: enough blocks for eight on every SM, else longer walks
+inline int stencil_cols(const GridDev &g) {
+  const int64_t rows = (g.ny + COLT - 1) / COLT;
+  return (int)std::max<int64_t>(1, rows * g.nx / (152 * 8));
 }
+inline dim3 stencil_grid(const GridDev &g, int ci) { return dim3((g.ny + COLT - 1) / COLT, (g.nx + ci - 1) / ci); }
 
 template <typename R>
 __global__ void __launch_bounds__(TPB) k_restrict(const StripDev *__restrict__ strips, int ny,
@@ -319,13 +389,25 @@ template void launch_strip_norms<double>(const StripDev *, int, int, const void 
 template void launch_strip_norms<float>(const StripDev *, int, int, const void *, double *, cudaStream_t);
 
 void launch_stencil(const GridDev &g, const double2 *x, double2 *y, cudaStream_t st) {
-  k_stencil<<<grid_for((int64_t)g.nx * g.ny), TPB, 0, st>>>(g, x, y);
+  const int ci = stencil_cols(g);
+  k_stencil_cols<false, false><<<stencil_grid(g, ci), COLT, 0, st>>>(g, x, nullptr, y, ci, nullptr);
   count_launch();
 }
-
 void launch_residual(const GridDev &g, const double2 *b, const double2 *x, double2 *r, cudaStream_t st) {
-  k_residual<<<grid_for((int64_t)g.nx * g.ny), TPB, 0, st>>>(g, b, x, r);
+  const int ci = stencil_cols(g);
+  k_stencil_cols<true, false><<<stencil_grid(g, ci), COLT, 0, st>>>(g, x, b, r, ci, nullptr);
   count_launch();
+}
+int64_t residual_norm_partials(const GridDev &g) {
+  const dim3 n = stencil_grid(g, stencil_cols(g));
+  return (int64_t)n.x * n.y;
+}
+void launch_residual_norm(const GridDev &g, const double2 *b, const double2 *x, double2 *r, double2 *partial,
+                          double2 *norms2, cudaStream_t st) {
+  const int ci = stencil_cols(g);
+  k_stencil_cols<true, true><<<stencil_grid(g, ci), COLT, 0, st>>>(g, x, b, r, ci, partial);
+  k_sum_pairs<<<1, TPB, 0, st>>>(partial, residual_norm_partials(g), norms2);
+  count_launch(2);
 }
 
 template <typename R>
