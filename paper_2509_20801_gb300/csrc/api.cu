@@ -81,6 +81,32 @@ struct DBuf {
   template <typename T> T *as() const { return reinterpret_cast<T *>(p); }
 };
 
+// owning page-locked host allocation (asynchronous copies in and out of it
+// do not stage)
+struct HBuf {
+  void *p = nullptr;
+  size_t bytes = 0;
+  HBuf() = default;
+  HBuf(const HBuf &) = delete;
+  HBuf &operator=(const HBuf &) = delete;
+  ~HBuf() {
+    if (p) cudaFreeHost(p);
+  }
+  void alloc(size_t n) {
+    if (n <= bytes) return;
+    if (p) cudaFreeHost(p);
+    p = nullptr;
+    bytes = 0;
+    if (cudaMallocHost(&p, n) != cudaSuccess) {
+      p = nullptr;
+      (void)cudaGetLastError();
+      throw std::bad_alloc();
+    }
+    bytes = n;
+  }
+  template <typename T> T *as() const { return reinterpret_cast<T *>(p); }
+};
+
 // SC-PML stretch on a line of n nodes (Eqs. 10-13): node u = 1..L of a PML
 // at depth (u - 1/2) cells, half node u + 1/2 at depth u cells from the
 // interface; sigma/(w eps0) = (m+1)(-ln R)/(2 k0 L delta) (rho/(L delta))^m.
@@ -240,6 +266,7 @@ struct stdd_ctx {
   DBuf d_guess, d_gscr;
   std::vector<double> lg_raw, lg_scaled;
   std::vector<int> lg_used;
+  HBuf h_krylov;      // the Gram-Schmidt coefficients and norms of a step, read back
   int V_cols = 0, V_rhs = 0;
   bool last_noconv = false;
   std::vector<std::vector<double>> history;
@@ -567,7 +594,8 @@ struct stdd_ctx {
   int sweep_flag_h = 0;
   void build_strip_levels();
   void poll_sweep_flag() {           // enqueue a copy of the flag (read after the next sync)
-    if (d_sweep_flag.p) CK(cudaMemcpyAsync(&sweep_flag_h, d_sweep_flag.p, sizeof(int), cudaMemcpyDeviceToHost, stream));
+    // (only persistent sweeps raise it; a copy into pageable memory waits for the stream)
+    if (d_sweep_flag.p && persistent_eff()) CK(cudaMemcpyAsync(&sweep_flag_h, d_sweep_flag.p, sizeof(int), cudaMemcpyDeviceToHost, stream));
   }
   void raise_sweep_flag() {          // after a sync: a persistent sweep gave up a barrier wait
     if (sweep_flag_h & 1) {
@@ -1754,8 +1782,9 @@ void stdd_ctx::gmres_multi(const stdd_solve_opts &o) {
   auto h1 = [&](int q) { return d_h.as<double2>() + (size_t)q * 2 * (m + 2); };
   auto h2 = [&](int q) { return h1(q) + (m + 2); };
   auto nrmq = [&](int q) { return nrm_base + 4 + 2 * q; };
+  h_krylov.alloc((size_t)(2 * (m + 2) + 1) * nq * sizeof(double2));
   struct St {
-    std::vector<cd> H, g, sn, hv;
+    std::vector<cd> H, g, sn;
     std::vector<double> cs;
     double bnorm = 0, nrm2 = 0, res = 0, tgt = 0;  // tgt: absolute residual target of the iteration
     int its = 0, reorth = 0, k = 0;
@@ -1768,7 +1797,6 @@ void stdd_ctx::gmres_multi(const stdd_solve_opts &o) {
     t.g.assign(m + 1, 0);
     t.sn.assign(m, 0);
     t.cs.assign(m, 0);
-    t.hv.assign(2 * (m + 2), 0);
     const double2 *b = d_b.as<double2>() + (int64_t)q * NN;
     t.bnorm = dev_norm(const_cast<double2 *>(b), NN, d_part, d_nrm, stream);
     t.tgt = o.rtol * t.bnorm;
@@ -1871,38 +1899,60 @@ void stdd_ctx::gmres_multi(const stdd_solve_opts &o) {
         pend(sp);
       }
       int sp = pbegin(PH_ORTHO);
-      for (int q : inner) {
-        double2 *w = V(q, j + 1);
-        stdd::launch_mdot(V(q, 0), n, j + 1, w, n, d_part.as<double2>(), h1(q), stream, 1);
-        stdd::launch_maxpy_norm(V(q, 0), n, j + 1, h1(q), w, n, part, nrmq(q), stream);
-        CK(cudaMemcpyAsync(S[q].hv.data(), h1(q), sizeof(double2) * (j + 2), cudaMemcpyDeviceToHost, stream));
-        CK(cudaMemcpyAsync(&S[q].nrm2, nrmq(q), sizeof(double), cudaMemcpyDeviceToHost, stream));
+      // one launch of each kind for (up to KRYLOV_BATCH) right-hand sides,
+      // their results read back together through pinned memory
+      const int64_t ldh = 2 * (m + 2);
+      auto batches = [&](const std::vector<int> &qs) {
+        std::vector<stdd::KrylovBatch> out;
+        for (size_t i = 0; i < qs.size(); i += stdd::KRYLOV_BATCH) {
+          stdd::KrylovBatch B = {};
+          for (size_t k = i; k < std::min(qs.size(), i + stdd::KRYLOV_BATCH); ++k) {
+            B.q[B.n] = qs[k];
+            B.off[B.n++] = V(qs[k], 0) - Vb;
+          }
+          out.push_back(B);
+        }
+        return out;
+      };
+      double2 *hh = h_krylov.as<double2>();
+      double *nh = reinterpret_cast<double *>(hh + (size_t)ldh * nq);
+      auto read_back = [&]() {
+        CK(cudaMemcpyAsync(hh, d_h.p, (size_t)ldh * nq * sizeof(double2), cudaMemcpyDeviceToHost, stream));
+        CK(cudaMemcpyAsync(nh, nrm_base + 4, 2 * (size_t)nq * sizeof(double), cudaMemcpyDeviceToHost, stream));
+      };
+      for (const stdd::KrylovBatch &B : batches(inner)) {
+        stdd::launch_mdot(B, Vb, n, j + 1, n, d_part.as<double2>(), h1(0), ldh, stream, 1);
+        stdd::launch_maxpy_norm(B, Vb, n, j + 1, h1(0), ldh, n, part, nrmq(0), 2, stream);
       }
+      read_back();
       poll_sweep_flag();
       CK(cudaStreamSynchronize(stream));
       raise_sweep_flag();
       std::vector<int> again;
       for (int q : inner) {
         St &t = S[q];
-        for (int i = 0; i <= j; ++i) t.H[(size_t)i * m + j] = t.hv[i];
-        if (t.nrm2 < 0.5 * t.hv[j + 1].real()) again.push_back(q);
+        t.nrm2 = nh[2 * q];
+        const cd *hv = reinterpret_cast<const cd *>(hh + q * ldh);
+        for (int i = 0; i <= j; ++i) t.H[(size_t)i * m + j] = hv[i];
+        if (t.nrm2 < 0.5 * hv[j + 1].real()) again.push_back(q);
       }
-      for (int q : again) {
-        double2 *w = V(q, j + 1);
-        stdd::launch_mdot(V(q, 0), n, j + 1, w, n, d_part.as<double2>(), h2(q), stream);
-        stdd::launch_maxpy_norm(V(q, 0), n, j + 1, h2(q), w, n, part, nrmq(q), stream);
-        CK(cudaMemcpyAsync(S[q].hv.data() + (m + 2), h2(q), sizeof(double2) * (j + 1), cudaMemcpyDeviceToHost,
-                           stream));
-        CK(cudaMemcpyAsync(&S[q].nrm2, nrmq(q), sizeof(double), cudaMemcpyDeviceToHost, stream));
+      if (!again.empty()) {
+        for (const stdd::KrylovBatch &B : batches(again)) {
+          stdd::launch_mdot(B, Vb, n, j + 1, n, d_part.as<double2>(), h2(0), ldh, stream);
+          stdd::launch_maxpy_norm(B, Vb, n, j + 1, h2(0), ldh, n, part, nrmq(0), 2, stream);
+        }
+        read_back();
+        CK(cudaStreamSynchronize(stream));
       }
-      if (!again.empty()) CK(cudaStreamSynchronize(stream));
       for (int q : again) {
         St &t = S[q];
-        for (int i = 0; i <= j; ++i) t.H[(size_t)i * m + j] += t.hv[(m + 2) + i];
+        t.nrm2 = nh[2 * q];
+        const cd *hv = reinterpret_cast<const cd *>(hh + q * ldh) + (m + 2);
+        for (int i = 0; i <= j; ++i) t.H[(size_t)i * m + j] += hv[i];
         ++t.reorth;
       }
       pend(sp);
-      std::vector<int> next;
+      std::vector<int> next, scaled;
       for (int q : inner) {
         St &t = S[q];
         std::vector<cd> &H = t.H;
@@ -1925,9 +1975,11 @@ void stdd_ctx::gmres_multi(const stdd_solve_opts &o) {
         history[q].push_back(est);
         if (!std::isfinite(est)) throw std::range_error("non-finite residual estimate");
         const bool breakdown = !(hn > 0) || std::abs(hjj) == 0;
-        if (!breakdown) stdd::launch_scale(V(q, j + 1), nrmq(q), V(q, j + 1), n, stream);
+        if (!breakdown) scaled.push_back(q);
         if (!(est * t.bnorm <= t.tgt || t.its >= o.maxit || breakdown)) next.push_back(q);
       }
+      for (const stdd::KrylovBatch &B : batches(scaled))
+        stdd::launch_scale_basis(B, Vb, n, j + 1, nrmq(0), 2, n, stream);
       inner.swap(next);
     }
     // x_q += Z_q y_q with y_q = R_q^-1 g_q

@@ -251,13 +251,25 @@ void launch_band_gather(const BandDev &b, int ny, const double2 *x, double2 *y, 
 void launch_band_scatter_add(const BandDev &b, int ny, const double2 *y, double2 *x, cudaStream_t st); // x += y
 
 // ---- Krylov kernels (kernels_krylov.cu), FP64 complex
-// partial[blk][i] = sum_g conj(V_i[g]) w[g], i < m; then h[i] = sum_blk partial.
-// With self_norm, h[m] = (||w||^2, 0) as well.
-void launch_mdot(const double2 *V, int64_t ldv, int m, const double2 *w, int64_t n, double2 *partial,
-                 double2 *h, cudaStream_t st, int self_norm = 0);
-// w -= sum_i h[i] V_i, and nrm2 = ||w||^2 (partials then a fixed-order sum)
-void launch_maxpy_norm(const double2 *V, int64_t ldv, int m, const double2 *h, double2 *w, int64_t n,
-                       double *partial, double *nrm2, cudaStream_t st);
+// The bases one launch works on: n of them, basis k of right-hand side q[k]
+// at V + off[k], its vectors ldv apart.  Every call of a step treats vector m
+// (the one being orthogonalised) of each against vectors 0 .. m - 1.
+constexpr int KRYLOV_BATCH = 16;
+struct KrylovBatch {
+  int n;
+  int q[KRYLOV_BATCH];
+  int64_t off[KRYLOV_BATCH];
+};
+// h[q ldh + i] = sum_g conj(V_i[g]) V_m[g], i < m; with self_norm, entry m is
+// (||V_m||^2, 0) as well.  partial: krylov_partial_blocks() * (m + 1) pairs.
+void launch_mdot(const KrylovBatch &B, const double2 *V, int64_t ldv, int m, int64_t n, double2 *partial, double2 *h,
+                 int64_t ldh, cudaStream_t st, int self_norm = 0);
+// V_m -= sum_i h[q ldh + i] V_i, nrm2[q ldn] = ||V_m||^2 (partials then a fixed-order sum)
+void launch_maxpy_norm(const KrylovBatch &B, double2 *V, int64_t ldv, int m, const double2 *h, int64_t ldh, int64_t n,
+                       double *partial, double *nrm2, int64_t ldn, cudaStream_t st);
+// V_m /= sqrt(nrm2[q ldn])
+void launch_scale_basis(const KrylovBatch &B, double2 *V, int64_t ldv, int m, const double *nrm2, int64_t ldn,
+                        int64_t n, cudaStream_t st);
 // x += sum_i y[i] Z_i
 void launch_maxpy(const double2 *Z, int64_t ldz, int m, const double2 *y, double2 *x, int64_t n,
                   cudaStream_t st);
