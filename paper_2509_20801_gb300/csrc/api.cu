@@ -2181,6 +2181,12 @@ template <typename F> stdd_status guarded(stdd_ctx *c, F &&f) {
 void copy_in(void *dst, const void *src, size_t bytes, int is_device, cudaStream_t st) {
   CK(cudaMemcpyAsync(dst, src, bytes, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
 }
+// device buffers the kernels can use where they are: aligned for double2 and
+// the output clear of the input whose neighbours other threads still read
+bool in_place(const double *in, const double *out, size_t bytes, int is_device) {
+  const uintptr_t a = reinterpret_cast<uintptr_t>(in), b = reinterpret_cast<uintptr_t>(out);
+  return is_device && a % sizeof(double2) == 0 && b % sizeof(double2) == 0 && (a + bytes <= b || b + bytes <= a);
+}
 void copy_out(void *dst, const void *src, size_t bytes, int is_device, cudaStream_t st) {
   CK(cudaMemcpyAsync(dst, src, bytes, is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -2420,6 +2426,12 @@ stdd_status stdd_apply_operator(stdd_ctx *c, const double *x, double *y, int is_
     if (!x || !y) throw ArgError("null vector");
     c->require_operator();
     const int64_t n = c->N();
+    if (in_place(x, y, n * sizeof(double2), is_device)) {
+      stdd::launch_stencil(c->grid(), reinterpret_cast<const double2 *>(x), reinterpret_cast<double2 *>(y), c->stream);
+      CK(cudaGetLastError());
+      CK(cudaStreamSynchronize(c->stream));
+      return;
+    }
     c->d_w.alloc(n * sizeof(double2));
     c->d_r.alloc(n * sizeof(double2));
     copy_in(c->d_w.p, x, n * sizeof(double2), is_device, c->stream);
@@ -2513,18 +2525,33 @@ stdd_status stdd_residual(stdd_ctx *c, const double *x, const double *b, double 
     if (!x || !b || !r || !rel_out) throw ArgError("null argument");
     c->require_operator();
     const int64_t n = c->N();
-    c->d_w.alloc(n * sizeof(double2));
-    c->d_r.alloc(n * sizeof(double2));
-    c->d_x.alloc(n * sizeof(double2));
-    c->d_part.alloc((size_t)stdd::krylov_partial_blocks() * sizeof(double2));
+    const size_t bytes = n * sizeof(double2);
+    const stdd::GridDev g = c->grid();
+    c->d_part.alloc((size_t)stdd::residual_norm_partials(g) * sizeof(double2));
     c->d_nrm.alloc(4 * sizeof(double));
-    copy_in(c->d_w.p, x, n * sizeof(double2), is_device, c->stream);
-    copy_in(c->d_x.p, b, n * sizeof(double2), is_device, c->stream);
-    stdd::launch_residual(c->grid(), c->d_x.as<double2>(), c->d_w.as<double2>(), c->d_r.as<double2>(), c->stream);
-    const double rn = dev_norm(c->d_r.as<double2>(), n, c->d_part, c->d_nrm, c->stream);
-    const double bn = dev_norm(c->d_x.as<double2>(), n, c->d_part, c->d_nrm, c->stream);
+    // r may be b's buffer; anything else that overlaps goes through copies
+    const bool direct = in_place(x, r, bytes, is_device) && (r == b || in_place(b, r, bytes, is_device)) &&
+                        reinterpret_cast<uintptr_t>(b) % sizeof(double2) == 0;
+    const double2 *xd = reinterpret_cast<const double2 *>(x), *bd = reinterpret_cast<const double2 *>(b);
+    double2 *rd = reinterpret_cast<double2 *>(r);
+    if (!direct) {
+      c->d_w.alloc(bytes);
+      c->d_r.alloc(bytes);
+      c->d_x.alloc(bytes);
+      copy_in(c->d_w.p, x, bytes, is_device, c->stream);
+      copy_in(c->d_x.p, b, bytes, is_device, c->stream);
+      xd = c->d_w.as<double2>();
+      bd = c->d_x.as<double2>();
+      rd = c->d_r.as<double2>();
+    }
+    stdd::launch_residual_norm(g, bd, xd, rd, c->d_part.as<double2>(), c->d_nrm.as<double2>(), c->stream);
+    CK(cudaGetLastError());
+    double n2[2] = {0, 0};
+    CK(cudaMemcpyAsync(n2, c->d_nrm.p, sizeof(n2), cudaMemcpyDeviceToHost, c->stream));
+    if (!direct) copy_out(r, rd, bytes, is_device, c->stream);
+    CK(cudaStreamSynchronize(c->stream));
+    const double rn = std::sqrt(n2[0]), bn = std::sqrt(n2[1]);
     *rel_out = bn > 0 ? rn / bn : rn;
-    copy_out(r, c->d_r.p, n * sizeof(double2), is_device, c->stream);
   });
 }
 
