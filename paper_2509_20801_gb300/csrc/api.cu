@@ -728,8 +728,8 @@ void stdd_ctx::factor() {
     else autotune<float>();
   }
   if (forced_split) {
-    // one split everywhere it is valid (32-row items for the grid split, at
-    // most MF_MAXSEG segments for an in-block one); results do not change
+    // one split everywhere it is valid (32-row items for the grid split, as
+    // many chains as a block holds for an in-block one); results do not change
     for (auto &li : levels) {
       auto pick = [&](int rows, int cols) {
         int sp = forced_split;
@@ -737,8 +737,7 @@ void stdd_ctx::factor() {
           if (rows == 32) return sp;
           sp = 8;
         }
-        if (sp > 256 / rows) sp = 256 / rows;
-        if (!stdd::mf_split_fits(elem() / 2, sp, cols)) sp = 1;
+        while (!stdd::mf_split_fits(elem(), rows, sp, cols)) sp /= 2;
         return sp;
       };
       li.split_up = li.split_up1 = pick(li.rows_up, li.max_p);
@@ -766,12 +765,13 @@ void stdd_ctx::build_strip_levels() {
       l.rows_down = li.rows_down;
       // (the persistent kernel splits within a block only; any split gives
       // the same sums)
-      auto inblock = [&](int sp, int cols) {
+      auto inblock = [&](int sp, int rows, int cols) {
         if (sp > 8) sp = 8;
-        return stdd::mf_split_fits(elem() / 2, sp, cols) ? sp : 1;
+        while (!stdd::mf_split_fits(elem(), rows, sp, cols)) sp /= 2;
+        return sp;
       };
-      l.split_up = inblock(li.split_up1, li.max_p);
-      l.split_down = inblock(li.split_down1, li.max_n);
+      l.split_up = inblock(li.split_up1, li.rows_up, li.max_p);
+      l.split_down = inblock(li.split_down1, li.rows_down, li.max_n);
       l.max_n = li.max_n;
       l.pad_ = 0;
     }
@@ -989,7 +989,7 @@ void stdd_ctx::build_structure() {
   auto pow2_split = [&](int cols, int rows) {
     int want = (cols + 4 * rows - 1) / (4 * rows), s = 1;
     while (s < want && s < 8) s *= 2;
-    if (!stdd::mf_split_fits(elem() / 2, s, cols)) s = 1;
+    while (!stdd::mf_split_fits(elem(), rows, s, cols)) s /= 2;
     return s;
   };
   std::vector<int2> items;
@@ -1145,11 +1145,9 @@ template <typename R> void stdd_ctx::autotune() {
             if (sp == stdd::MF_SPLIT_GRID) {
               if (rows != 32 || cols <= stdd::MF_SEG) break;
             } else {
-              if (sp > 256 / rows) continue;
-              if (!stdd::mf_split_fits(sizeof(R), sp, cols)) continue;
-              // more sharers than shares leave warps without work
-              const int share = sizeof(R) == 8 ? stdd::MF_SUB : stdd::MF_SEG;
-              if (sp > 1 && (sp / 2) * share >= cols) continue;
+              if (!stdd::mf_split_fits(2 * sizeof(R), rows, sp, cols)) continue;
+              // more sharers than chains leave row groups without work
+              if (sp > 1 && (sp / 2) * stdd::MF_SUB >= cols) continue;
             }
             float ms_min = 1e30f;
             for (int rep = 0; rep < 3; ++rep) {

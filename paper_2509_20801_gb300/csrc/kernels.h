@@ -15,17 +15,22 @@ constexpr int MF_NB = 32;             // pivot block of the blocked Gauss-Jordan
 constexpr int MF_PANEL_THREADS = 128; // rows / columns per panel tile
 constexpr int MF_SMALL = 64;          // fronts with n <= MF_SMALL are swept in shared memory
 constexpr int MF_SEG = 128;           // columns per fixed summation segment of the sweeps
-constexpr int MF_MAXSEG = 16;         // segments an item may have when its columns are split
 constexpr int MF_SPLIT_GRID = 16;     // split value: one warp per (item, sub-segment) anywhere in the grid
 constexpr int MF_SUB = 32;            // columns per chain inside a segment (segment = chains added in order)
 static_assert(MF_SEG % MF_SUB == 0, "segments are whole sub-segments");
-constexpr int MF_MAXCHAIN = 64;       // complex128: chains a block's items may have in all when split
-// whether items of `cols` columns may share them among `split` row groups (complex64: whole segments) or
-// warps (complex128: whole chains) of a block; real: bytes of a real number
-inline bool mf_split_fits(size_t real, int split, int cols) {
-  if (split <= 1) return true;
-  return real == 8 ? (cols + MF_SUB - 1) / MF_SUB <= MF_MAXCHAIN * split / 8
-                   : (cols + MF_SEG - 1) / MF_SEG <= MF_MAXSEG;
+constexpr int MF_PART_BYTES = 32 << 10;   // shared memory of a block's split items' chain sums
+// chains an item may have when `split` row groups (complex64: `rows` lanes)
+// or warps (complex128) of a 256-thread block share its columns, for nr
+// right-hand sides at a time; value: bytes of a complex number
+constexpr int mf_block_items(int value, int rows) { return value == 16 ? 8 : 256 / rows; }
+constexpr __host__ __device__ int mf_max_chains(int value, int rows, int split, int nr) {
+  const int items = (value == 16 ? 8 : 256 / rows) / split;
+  // a complex128 warp's lanes hold two components of 16 rows, or of 32 in two rounds
+  return MF_PART_BYTES / (items * nr * rows * value);
+}
+inline bool mf_split_fits(size_t value, int rows, int split, int cols, int nr = 1) {
+  return split <= 1 || (split <= mf_block_items((int)value, rows) &&
+                        (cols + MF_SUB - 1) / MF_SUB <= mf_max_chains((int)value, rows, split, nr));
 }
 
 // Everything a multifrontal kernel needs (device pointers).

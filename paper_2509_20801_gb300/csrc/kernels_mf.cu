@@ -903,32 +903,27 @@ template <int W, typename C> __device__ __forceinline__ C shfl_w(unsigned mask, 
   return v;
 }
 
-// acc[q] = sum over columns [c0, c1) of M(r, c) * vec_q(c), q < NR, for one
-// segment; M(r, c) at M[c * ld + r]; vec_q(c) comes from gather(c, q).
-// Each matrix entry is loaded once for all NR right-hand sides.
-template <int ROWS, int NR, typename C, typename Gather>
-__device__ __forceinline__ void seg_dot(const C *__restrict__ M, int64_t ld, int r, bool row, int c0, int c1,
-                                        int lane, unsigned mask, Gather gather, C (&acc)[NR]) {
+// Sums over the chains [k0, k1) (MF_SUB columns each, the last one up to
+// cend) of M(r, c) * vec_q(c), q < NR; M(r, c) at M[c * ld + r]; vec_q(c)
+// comes from gather(c, q); sink(k, s) receives chain k's sums.  Each matrix
+// entry is loaded once for all NR right-hand sides.
+template <int ROWS, int NR, typename C, typename Gather, typename Sink>
+__device__ __forceinline__ void row_chains(const C *__restrict__ M, int64_t ld, int r, bool row, int k0, int k1,
+                                           int cend, int lane, unsigned mask, Gather gather, Sink sink) {
   // the next chunk's vector values are requested before this chunk's
   // products (at the top tree levels a few warps carry a whole phase and
   // would otherwise wait for the dependent gather once per chunk)
   constexpr int U = NR > 1 ? (32 / NR > 4 ? 32 / NR : 4) : 32;
   constexpr int UU = U < ROWS ? U : ROWS;
-  static_assert(MF_SUB % ROWS == 0, "a sub-segment is a whole number of chunks");
-  // each MF_SUB columns form a chain of their own (sub), folded into the
-  // segment sum in column order: acc = ((s0 + s1) + s2) + s3
-  C sub[NR];
+  static_assert(MF_SUB % ROWS == 0, "a chain is a whole number of chunks");
+  const int c0 = k0 * MF_SUB, c1 = min(cend, k1 * MF_SUB);
+  C sub[NR], vn[NR], m[UU];
 #pragma unroll
-  for (int q = 0; q < NR; ++q) acc[q] = sub[q] = czero<C>();
-  C vn[NR];
-#pragma unroll
-  for (int q = 0; q < NR; ++q) vn[q] = c0 + lane < c1 ? gather(c0 + lane, q) : czero<C>();
-  C m[UU];
+  for (int q = 0; q < NR; ++q) {
+    sub[q] = czero<C>();
+    vn[q] = c0 + lane < c1 ? gather(c0 + lane, q) : czero<C>();
+  }
   for (int cb = c0; cb < c1; cb += ROWS) {
-    if ((cb - c0) % MF_SUB == 0) {
-#pragma unroll
-      for (int q = 0; q < NR; ++q) sub[q] = czero<C>();
-    }
     C v[NR];
 #pragma unroll
     for (int q = 0; q < NR; ++q) v[q] = vn[q];
@@ -964,10 +959,10 @@ __device__ __forceinline__ void seg_dot(const C *__restrict__ M, int64_t ld, int
         for (int q = 0; q < NR; ++q) sub[q] = cfma(m, shfl_w<ROWS>(mask, v[q], u), sub[q]);
       }
     }
-    if ((cb + ROWS - c0) % MF_SUB == 0 || cb + ROWS >= c1) {
-      const bool first = cb - c0 < MF_SUB;
+    if ((cb + ROWS) % MF_SUB == 0 || cb + ROWS >= c1) {
+      sink(cb / MF_SUB, sub);
 #pragma unroll
-      for (int q = 0; q < NR; ++q) acc[q] = first ? sub[q] : cadd(acc[q], sub[q]);
+      for (int q = 0; q < NR; ++q) sub[q] = czero<C>();
     }
   }
 }
@@ -1200,6 +1195,17 @@ __global__ void __launch_bounds__(256) mf_up_gather(MfArgs a, int f0, int nf, in
 // themselves (WSrc, the gather's own arithmetic), the front's first row
 // chunk stores w_p for the way down, and each row starts from the
 // children's update vectors.
+// Chain sums fold four to a segment sum, segment sums onto the total in
+// column order, whichever row group computed them.
+template <typename C, int NR> struct ChainFold {
+  C total[NR], seg[NR];
+  __device__ __forceinline__ void add(int q, int k, int nk, C s) {
+    constexpr int PER = MF_SEG / MF_SUB;
+    seg[q] = k % PER == 0 ? s : cadd(seg[q], s);
+    if (k % PER == PER - 1 || k == nk - 1) total[q] = cadd(total[q], seg[q]);
+  }
+};
+
 template <typename R, int ROWS, int NR, bool FUSED = false>
 __device__ __forceinline__ void up_block(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                          int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
@@ -1211,7 +1217,8 @@ __device__ __forceinline__ void up_block(const MfArgs &a, const int2 *__restrict
   const int it = vb * ipc + il;
   const bool active = it < nitems;
   const unsigned mask = ROWS == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
-  int p = 0, b = 0, r = 0, seg0 = 0, seg1 = 0, nseg = 0;
+  const int nkmax = mf_max_chains(8, ROWS, split, NR);
+  int p = 0, b = 0, r = 0, k0 = 0, k1 = 0, nk = 0;
   bool row = false;
   const C *G = nullptr;
   const int *nodes = nullptr, *pc = nullptr;
@@ -1235,21 +1242,21 @@ __device__ __forceinline__ void up_block(const MfArgs &a, const int2 *__restrict
     nodes = a.nodes + f.node_off;
     u = reinterpret_cast<C *>(a.ub_cur) + f.u_off * nrhs;
     if (a.pcol) pc = a.pcol + f.piv_off;
-    nseg = (p + MF_SEG - 1) / MF_SEG;
-    seg0 = sidx * nseg / split;
-    seg1 = (sidx + 1) * nseg / split;
+    nk = (p + MF_SUB - 1) / MF_SUB;
+    k0 = sidx * nk / split;
+    k1 = (sidx + 1) * nk / split;
   }
   C *wl = reinterpret_cast<C *>(a.wloc);
-  for (int q0 = 0; q0 < nrhs; q0 += NR) {
-    C total[NR];
+  C *mine = part + (int64_t)il * nkmax * NR * ROWS + lane;
+  for (int q0 = blockIdx.y * NR; q0 < nrhs; q0 += gridDim.y * NR) {
+    ChainFold<C, NR> fold;
 #pragma unroll
-    for (int q = 0; q < NR; ++q) total[q] = czero<C>();
-    if (active) {
-      if (row && sidx == 0)
-#pragma unroll
-        for (int q = 0; q < NR; ++q)
-          if (q0 + q < nrhs)
-            total[q] = FUSED ? wsrc_children(src, p + r, q0 + q, czero<C>()) : u[(int64_t)(q0 + q) * b + r];
+    for (int q = 0; q < NR; ++q) {
+      fold.total[q] = fold.seg[q] = czero<C>();
+      if (row && sidx == 0 && q0 + q < nrhs)
+        fold.total[q] = FUSED ? wsrc_children(src, p + r, q0 + q, czero<C>()) : u[(int64_t)(q0 + q) * b + r];
+    }
+    if (k0 < k1) {
       auto gather = [&](int j, int q) {
         if (q0 + q >= nrhs) return czero<C>();
         if (!FUSED) return wl[(q0 + q) * ldt + voff + nodes[pc ? pc[j] : j]];
@@ -1258,29 +1265,23 @@ __device__ __forceinline__ void up_block(const MfArgs &a, const int2 *__restrict
         if (writer) wl[gi] = w;
         return w;
       };
-      for (int sg = seg0; sg < seg1; ++sg) {
-        C sv[NR];
-        seg_dot<ROWS, NR, C>(G, b, r, row, sg * MF_SEG, min(p, (sg + 1) * MF_SEG), lane, mask, gather, sv);
-        if (split == 1) {
+      row_chains<ROWS, NR, C>(G, b, r, row, k0, k1, p, lane, mask, gather, [&](int k, const C(&s)[NR]) {
 #pragma unroll
-          for (int q = 0; q < NR; ++q) total[q] = cadd(total[q], sv[q]);
-        } else {
-          part[(il * MF_MAXSEG + sg) * ROWS + lane] = sv[0];
-        }
+        for (int q = 0; q < NR; ++q)
+          if (split == 1) fold.add(q, k, nk, s[q]);
+          else mine[(k * NR + q) * ROWS] = s[q];
+      });
+    }
+    if (split > 1) __syncthreads();
+    if (active && row && sidx == 0) {
+#pragma unroll
+      for (int q = 0; q < NR; ++q) {
+        if (split > 1)
+          for (int k = 0; k < nk; ++k) fold.add(q, k, nk, mine[(k * NR + q) * ROWS]);
+        if (q0 + q < nrhs) u[(int64_t)(q0 + q) * b + r] = fold.total[q];
       }
     }
-    if (split > 1) {
-      __syncthreads();
-      if (active && row && sidx == 0) {
-        for (int sg = 0; sg < nseg; ++sg) total[0] = cadd(total[0], part[(il * MF_MAXSEG + sg) * ROWS + lane]);
-        u[(int64_t)q0 * b + r] = total[0];
-      }
-      __syncthreads();
-    } else if (active && row) {
-#pragma unroll
-      for (int q = 0; q < NR; ++q)
-        if (q0 + q < nrhs) u[(int64_t)(q0 + q) * b + r] = total[q];
-    }
+    if (split > 1) __syncthreads();
   }
 }
 
@@ -1298,7 +1299,8 @@ __device__ __forceinline__ void down_block(const MfArgs &a, const int2 *__restri
   const int it = vb * ipc + il;
   const bool active = it < nitems;
   const unsigned mask = ROWS == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
-  int p = 0, n = 0, r = 0, seg0 = 0, seg1 = 0, nseg = 0;
+  const int nkmax = mf_max_chains(8, ROWS, split, NR);
+  int p = 0, n = 0, r = 0, k0 = 0, k1 = 0, nk = 0;
   bool row = false;
   const C *Fm = nullptr;
   const int *nodes = nullptr, *pc = nullptr;
@@ -1314,45 +1316,40 @@ __device__ __forceinline__ void down_block(const MfArgs &a, const int2 *__restri
     row = r < p;
     nodes = a.nodes + f.node_off;
     if (a.pcol) pc = a.pcol + f.piv_off;
-    nseg = (n + MF_SEG - 1) / MF_SEG;
-    seg0 = sidx * nseg / split;
-    seg1 = (sidx + 1) * nseg / split;
+    nk = (n + MF_SUB - 1) / MF_SUB;
+    k0 = sidx * nk / split;
+    k1 = (sidx + 1) * nk / split;
   }
   C *tv = reinterpret_cast<C *>(a.tloc);
   const C *wl = reinterpret_cast<const C *>(a.wloc);
-  for (int q0 = 0; q0 < nrhs; q0 += NR) {
-    C total[NR];
+  C *mine = part + (int64_t)il * nkmax * NR * ROWS + lane;
+  for (int q0 = blockIdx.y * NR; q0 < nrhs; q0 += gridDim.y * NR) {
+    ChainFold<C, NR> fold;
 #pragma unroll
-    for (int q = 0; q < NR; ++q) total[q] = czero<C>();
-    if (active) {
+    for (int q = 0; q < NR; ++q) fold.total[q] = fold.seg[q] = czero<C>();
+    if (k0 < k1) {
       auto gather = [&](int c, int q) {
         if (q0 + q >= nrhs) return czero<C>();
         const int64_t base = (q0 + q) * ldt + voff;
         return c < p ? wl[base + nodes[pc ? pc[c] : c]] : cneg(tv[base + nodes[c]]);
       };
-      for (int sg = seg0; sg < seg1; ++sg) {
-        C sv[NR];
-        seg_dot<ROWS, NR, C>(Fm, p, r, row, sg * MF_SEG, min(n, (sg + 1) * MF_SEG), lane, mask, gather, sv);
-        if (split == 1) {
+      row_chains<ROWS, NR, C>(Fm, p, r, row, k0, k1, n, lane, mask, gather, [&](int k, const C(&s)[NR]) {
 #pragma unroll
-          for (int q = 0; q < NR; ++q) total[q] = cadd(total[q], sv[q]);
-        } else {
-          part[(il * MF_MAXSEG + sg) * ROWS + lane] = sv[0];
-        }
+        for (int q = 0; q < NR; ++q)
+          if (split == 1) fold.add(q, k, nk, s[q]);
+          else mine[(k * NR + q) * ROWS] = s[q];
+      });
+    }
+    if (split > 1) __syncthreads();
+    if (active && row && sidx == 0) {
+#pragma unroll
+      for (int q = 0; q < NR; ++q) {
+        if (split > 1)
+          for (int k = 0; k < nk; ++k) fold.add(q, k, nk, mine[(k * NR + q) * ROWS]);
+        if (q0 + q < nrhs) tv[(q0 + q) * ldt + voff + nodes[r]] = fold.total[q];
       }
     }
-    if (split > 1) {
-      __syncthreads();
-      if (active && row && sidx == 0) {
-        for (int sg = 0; sg < nseg; ++sg) total[0] = cadd(total[0], part[(il * MF_MAXSEG + sg) * ROWS + lane]);
-        tv[q0 * ldt + voff + nodes[r]] = total[0];
-      }
-      __syncthreads();
-    } else if (active && row) {
-#pragma unroll
-      for (int q = 0; q < NR; ++q)
-        if (q0 + q < nrhs) tv[(q0 + q) * ldt + voff + nodes[r]] = total[q];
-    }
+    if (split > 1) __syncthreads();
   }
 }
 
@@ -1415,8 +1412,8 @@ __device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restr
     k1 = (sidx + 1) * nk / split;
   }
   double2 *wl = reinterpret_cast<double2 *>(a.wloc);
-  double *mine = part + (int64_t)il * (MF_MAXCHAIN * split / 8) * MT * 32 + lane;
-  for (int q0 = 0; q0 < nrhs; q0 += NR) {
+  double *mine = part + (int64_t)il * mf_max_chains(16, 16 * MT, split, NR) * NR * MT * 32 + lane;
+  for (int q0 = blockIdx.y * NR; q0 < nrhs; q0 += gridDim.y * NR) {
     FxRows<MT> f;
     f.start(G, E, r0, b, k0 * FX_COLS, min(p, k1 * FX_COLS), lane);
     if (PDL) level_wait();
@@ -1446,12 +1443,10 @@ __device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restr
                         [&](int k, const double(&s)[NR][MT]) {
 #pragma unroll
                           for (int t = 0; t < MT; ++t)
-                            if (split == 1) {
 #pragma unroll
-                              for (int q = 0; q < NR; ++q) fold.add(q, t, k, nk, s[q][t]);
-                            } else {
-                              mine[(k * MT + t) * 32] = s[0][t];
-                            }
+                            for (int q = 0; q < NR; ++q)
+                              if (split == 1) fold.add(q, t, k, nk, s[q][t]);
+                              else mine[((k * NR + q) * MT + t) * 32] = s[q][t];
                         });
     }
     if (split > 1) __syncthreads();
@@ -1460,7 +1455,9 @@ __device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restr
       for (int t = 0; t < MT; ++t) {
         const int r = r0 + 16 * t + fx_row(lane);
         if (split > 1)
-          for (int k = 0; k < nk; ++k) fold.add(0, t, k, nk, mine[(k * MT + t) * 32]);
+          for (int k = 0; k < nk; ++k)
+#pragma unroll
+            for (int q = 0; q < NR; ++q) fold.add(q, t, k, nk, mine[((k * NR + q) * MT + t) * 32]);
         if (r < b)
 #pragma unroll
           for (int q = 0; q < NR; ++q)
@@ -1503,8 +1500,8 @@ __device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__res
   }
   double2 *tv = reinterpret_cast<double2 *>(a.tloc);
   const double2 *wl = reinterpret_cast<const double2 *>(a.wloc);
-  double *mine = part + (int64_t)il * (MF_MAXCHAIN * split / 8) * MT * 32 + lane;
-  for (int q0 = 0; q0 < nrhs; q0 += NR) {
+  double *mine = part + (int64_t)il * mf_max_chains(16, 16 * MT, split, NR) * NR * MT * 32 + lane;
+  for (int q0 = blockIdx.y * NR; q0 < nrhs; q0 += gridDim.y * NR) {
     FxRows<MT> f;
     f.start(Fm, E, r0, p, k0 * FX_COLS, min(n, k1 * FX_COLS), lane);
     if (PDL) level_wait();
@@ -1521,12 +1518,10 @@ __device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__res
                         [&](int k, const double(&s)[NR][MT]) {
 #pragma unroll
                           for (int t = 0; t < MT; ++t)
-                            if (split == 1) {
 #pragma unroll
-                              for (int q = 0; q < NR; ++q) fold.add(q, t, k, nk, s[q][t]);
-                            } else {
-                              mine[(k * MT + t) * 32] = s[0][t];
-                            }
+                            for (int q = 0; q < NR; ++q)
+                              if (split == 1) fold.add(q, t, k, nk, s[q][t]);
+                              else mine[((k * NR + q) * MT + t) * 32] = s[q][t];
                         });
     }
     if (split > 1) __syncthreads();
@@ -1535,7 +1530,9 @@ __device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__res
       for (int t = 0; t < MT; ++t) {
         const int r = r0 + 16 * t + fx_row(lane);
         if (split > 1)
-          for (int k = 0; k < nk; ++k) fold.add(0, t, k, nk, mine[(k * MT + t) * 32]);
+          for (int k = 0; k < nk; ++k)
+#pragma unroll
+            for (int q = 0; q < NR; ++q) fold.add(q, t, k, nk, mine[((k * NR + q) * MT + t) * 32]);
         if (r < p)
 #pragma unroll
           for (int q = 0; q < NR; ++q)
@@ -1556,12 +1553,12 @@ template <typename R> __host__ __device__ constexpr int block_items(int rows) {
 // one (virtual) block of products of either precision; `part` holds the
 // segment sums of split items, the warps' vector words follow it
 template <typename R, int NR>
-constexpr int SWEEP_SMEM = MF_MAXSEG * 256 / 2 + (sizeof(R) == 8 ? 8 * NR * FX_COLS : 0);
+constexpr int SWEEP_SMEM = MF_PART_BYTES / (2 * sizeof(R)) + (sizeof(R) == 8 ? 8 * NR * FX_COLS : 0);
 template <typename R, int ROWS, int NR, bool FUSED, bool PDL>
 __device__ __forceinline__ void up_any(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                        int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
   if constexpr (sizeof(R) == 8) {
-    auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_MAXSEG * 256 / 2) + (threadIdx.x >> 5) * NR;
+    auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_PART_BYTES / sizeof(double2)) + (threadIdx.x >> 5) * NR;
     up_block_fx<ROWS / 16, NR, FUSED, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs);
   } else {
     if (PDL) level_wait();
@@ -1572,7 +1569,7 @@ template <typename R, int ROWS, int NR, bool PDL>
 __device__ __forceinline__ void down_any(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                          int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
   if constexpr (sizeof(R) == 8) {
-    auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_MAXSEG * 256 / 2) + (threadIdx.x >> 5) * NR;
+    auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_PART_BYTES / sizeof(double2)) + (threadIdx.x >> 5) * NR;
     down_block_fx<ROWS / 16, NR, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs);
   } else {
     if (PDL) level_wait();
@@ -1654,10 +1651,9 @@ __global__ void __launch_bounds__(256) mf_seg_partial(MfArgs a, const int2 *__re
                       out[32] = s[0][1];
                     });
   } else {
-    C sv[1];
     level_wait();
-    seg_dot<32, 1, C>(M, ld, r, row, c0, c1, lane, 0xffffffffu, gather, sv);
-    reinterpret_cast<C *>(a.segpart)[u * 32 + lane] = sv[0];
+    row_chains<32, 1, C>(M, ld, r, row, sg, sg + 1, cols, lane, 0xffffffffu, gather,
+                         [&](int, const C(&s)[1]) { reinterpret_cast<C *>(a.segpart)[u * 32 + lane] = s[0]; });
   }
 }
 
@@ -1695,9 +1691,9 @@ __global__ void __launch_bounds__(256) mf_seg_reduce(MfArgs a, const int2 *__res
 // 256-thread blocks that may start before the stream's previous kernel ends
 // (the kernel calls level_wait before it reads what that one writes)
 template <typename... P, typename... A>
-void launch_overlapped(void (*kernel)(P...), unsigned grid, cudaStream_t st, A... args) {
+void launch_overlapped(void (*kernel)(P...), dim3 grid, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(256);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -1925,24 +1921,32 @@ void mf_up_gather_level(const MfArgs &a, const LevelInfo &L, int nrhs, int64_t l
   count_launch();
 }
 
+// Groups of nr right-hand sides: one after another in the same blocks where
+// those fill the GPU (two blocks an SM; the second group finds the factors in
+// L1 or L2), side by side at the levels near the root, where a few items
+// alone leave it idle.
+static dim3 rhs_grid(int blocks, int nrhs, int nr) {
+  return dim3(blocks, blocks >= 2 * 152 ? 1 : (nrhs + nr - 1) / nr);
+}
+
 template <typename R>
 void mf_up_level(const MfArgs &a, const int2 *items, int nitems, int rows, int split, int nrhs, int64_t ldt,
                  cudaStream_t st, int cols_max, bool fused) {
   if (nitems == 0) return;
-  if (nrhs > 1) split = 1;  // several right-hand sides: every group keeps its segments in registers
+  constexpr int MAXR = sizeof(R) == 4 ? 4 : 2;   // right-hand sides per factor read
+  const int nr = (nrhs >= 4 && MAXR == 4) ? 4 : (nrhs >= 2 ? 2 : 1);
   if (split == MF_SPLIT_GRID) {
-    if (rows == 32 && a.segpart && cols_max > 0) {
+    if (nrhs == 1 && rows == 32 && a.segpart && cols_max > 0) {
       if (fused) mf_seg_launch<R, true, true>(a, items, nitems, cols_max, ldt, st);
       else mf_seg_launch<R, true, false>(a, items, nitems, cols_max, ldt, st);
       return;
     }
-    split = 1;
+    split = nrhs == 1 ? 1 : 8;   // as wide within a block, for every right-hand side
   }
-  if (cols_max > 0 && !mf_split_fits(sizeof(R), split, cols_max)) split = 1;
+  if (cols_max > 0)
+    while (!mf_split_fits(2 * sizeof(R), rows, split, cols_max, nr)) split /= 2;
   const int ipc = block_items<R>(rows) / split;
-  const int grid = (nitems + ipc - 1) / ipc;
-  constexpr int MAXR = sizeof(R) == 4 ? 4 : 2;   // right-hand sides per factor read
-  const int nr = (nrhs >= 4 && MAXR == 4) ? 4 : (nrhs >= 2 ? 2 : 1);
+  const dim3 grid = rhs_grid((nitems + ipc - 1) / ipc, nrhs, nr);
 #define STDD_UP(RW, NRV)                                                                \
   do {                                                                                  \
     if (fused) launch_overlapped(mf_up<R, RW, NRV, true>, grid, st, a, items, nitems, split, nrhs, ldt);  \
@@ -1961,19 +1965,19 @@ template <typename R>
 void mf_down_level(const MfArgs &a, const int2 *items, int nitems, int rows, int split, int nrhs, int64_t ldt,
                    cudaStream_t st, int cols_max) {
   if (nitems == 0) return;
-  if (nrhs > 1) split = 1;
+  constexpr int MAXR = sizeof(R) == 4 ? 4 : 2;   // right-hand sides per factor read
+  const int nr = (nrhs >= 4 && MAXR == 4) ? 4 : (nrhs >= 2 ? 2 : 1);
   if (split == MF_SPLIT_GRID) {
-    if (rows == 32 && a.segpart && cols_max > 0) {
+    if (nrhs == 1 && rows == 32 && a.segpart && cols_max > 0) {
       mf_seg_launch<R, false>(a, items, nitems, cols_max, ldt, st);
       return;
     }
-    split = 1;
+    split = nrhs == 1 ? 1 : 8;   // as wide within a block, for every right-hand side
   }
-  if (cols_max > 0 && !mf_split_fits(sizeof(R), split, cols_max)) split = 1;
+  if (cols_max > 0)
+    while (!mf_split_fits(2 * sizeof(R), rows, split, cols_max, nr)) split /= 2;
   const int ipc = block_items<R>(rows) / split;
-  const int grid = (nitems + ipc - 1) / ipc;
-  constexpr int MAXR = sizeof(R) == 4 ? 4 : 2;   // right-hand sides per factor read
-  const int nr = (nrhs >= 4 && MAXR == 4) ? 4 : (nrhs >= 2 ? 2 : 1);
+  const dim3 grid = rhs_grid((nitems + ipc - 1) / ipc, nrhs, nr);
 #define STDD_DOWN(RW, NRV) launch_overlapped(mf_down<R, RW, NRV>, grid, st, a, items, nitems, split, nrhs, ldt)
   if (rows == 16) {
     if (nr == 4) STDD_DOWN(16, MAXR); else if (nr == 2) STDD_DOWN(16, 2); else STDD_DOWN(16, 1);
