@@ -123,42 +123,41 @@ __device__ __forceinline__ C front_entry(const MfArgs &a, const FrontDev &f, con
                                          const bool *has, int r, int c) {
   const int p = f.p, H = s.y1 - s.y0;   // local box height
   double2 v = make_double2(0.0, 0.0);
-  if ((r < p || c < p) && a.sym) {
-    // row u of D A: the diagonal times d_u = s_x s_y; each coupling between
-    // two nodes computed from the lower-indexed node of the pair, so that
-    // entries (u, w) and (w, u) are the same number
-    const int u = a.nodes[f.node_off + r], w = a.nodes[f.node_off + c];
+  const int u = a.nodes[f.node_off + r], w = a.nodes[f.node_off + c], d = w - u;
+  // most entries couple no neighbours: decided before any division
+  if ((r < p || c < p) && (d == 0 || d == 1 || d == -1 || d == H || d == -H)) {
     const int ux = u / H, uy = u - ux * H;
-    const double2 sxu = a.lsx[s.coef_off + ux], syu = a.lsy[s.ycoef_off + uy];
-    if (u == w) {
-      const double2 xm = a.cxm[s.coef_off + ux], xp = a.cxp[s.coef_off + ux];
-      const double2 ym = a.cym[s.ycoef_off + uy], yp = a.cyp[s.ycoef_off + uy];
-      double2 d0;
-      d0.x = a.k0sq * a.eps[(int64_t)(s.x0 + ux) * a.H + s.y0 + uy] - xm.x - xp.x - ym.x - yp.x;
-      d0.y = -xm.y - xp.y - ym.y - yp.y;
-      v = cmul(cmul(sxu, syu), d0);
-    } else if (w == u - H || w == u + H) {
-      const int lx = w == u - H ? ux - 1 : ux;     // the pair's left column
-      v = cmul(cmul(a.lsx[s.coef_off + lx], a.cxp[s.coef_off + lx]), syu);
-    } else if ((w == u - 1 && uy > 0) || (w == u + 1 && uy < H - 1)) {
-      const int ly = w == u - 1 ? uy - 1 : uy;     // the pair's lower row
-      v = cmul(cmul(a.lsy[s.ycoef_off + ly], a.cyp[s.ycoef_off + ly]), sxu);
-    }
-  } else if (r < p || c < p) {
-    const int u = a.nodes[f.node_off + r], w = a.nodes[f.node_off + c];
-    const int ux = u / H, uy = u - ux * H;
-    if (u == w) {
+    if (a.sym) {
+      // row u of D A: the diagonal times d_u = s_x s_y; each coupling between
+      // two nodes computed from the lower-indexed node of the pair, so that
+      // entries (u, w) and (w, u) are the same number
+      const double2 sxu = a.lsx[s.coef_off + ux], syu = a.lsy[s.ycoef_off + uy];
+      if (d == 0) {
+        const double2 xm = a.cxm[s.coef_off + ux], xp = a.cxp[s.coef_off + ux];
+        const double2 ym = a.cym[s.ycoef_off + uy], yp = a.cyp[s.ycoef_off + uy];
+        double2 d0;
+        d0.x = a.k0sq * a.eps[(int64_t)(s.x0 + ux) * a.H + s.y0 + uy] - xm.x - xp.x - ym.x - yp.x;
+        d0.y = -xm.y - xp.y - ym.y - yp.y;
+        v = cmul(cmul(sxu, syu), d0);
+      } else if (d == -H || d == H) {
+        const int lx = d == -H ? ux - 1 : ux;     // the pair's left column
+        v = cmul(cmul(a.lsx[s.coef_off + lx], a.cxp[s.coef_off + lx]), syu);
+      } else if ((d == -1 && uy > 0) || (d == 1 && uy < H - 1)) {
+        const int ly = d == -1 ? uy - 1 : uy;     // the pair's lower row
+        v = cmul(cmul(a.lsy[s.ycoef_off + ly], a.cyp[s.ycoef_off + ly]), sxu);
+      }
+    } else if (d == 0) {
       const double2 xm = a.cxm[s.coef_off + ux], xp = a.cxp[s.coef_off + ux];
       const double2 ym = a.cym[s.ycoef_off + uy], yp = a.cyp[s.ycoef_off + uy];
       v.x = a.k0sq * a.eps[(int64_t)(s.x0 + ux) * a.H + s.y0 + uy] - xm.x - xp.x - ym.x - yp.x;
       v.y = -xm.y - xp.y - ym.y - yp.y;
-    } else if (w == u - H) {
+    } else if (d == -H) {
       v = a.cxm[s.coef_off + ux];
-    } else if (w == u + H) {
+    } else if (d == H) {
       v = a.cxp[s.coef_off + ux];
-    } else if (w == u - 1 && uy > 0) {
+    } else if (d == -1 && uy > 0) {
       v = a.cym[s.ycoef_off + uy];
-    } else if (w == u + 1 && uy < H - 1) {
+    } else if (d == 1 && uy < H - 1) {
       v = a.cyp[s.ycoef_off + uy];
     }
   }
@@ -182,7 +181,6 @@ __global__ void __launch_bounds__(256) mf_assemble(MfArgs a, int f0) {
   const FrontDev f = a.fronts[f0 + blockIdx.x];
   const int n = f.p + f.b;
   if (n <= MF_SMALL) return;
-  const int64_t nn = (int64_t)n * n;
   const StripDev s = a.strips[f.strip];
   FrontDev ch[2];
   bool has[2];
@@ -191,9 +189,13 @@ __global__ void __launch_bounds__(256) mf_assemble(MfArgs a, int f0) {
     has[ci] = f.child[ci] >= 0;
     if (has[ci]) ch[ci] = a.fronts[f.child[ci]];
   }
-  for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < nn; e += (int64_t)gridDim.y * blockDim.x) {
-    const int c = (int)(e / n), r = (int)(e - (int64_t)c * n);
-    st_elem<C>(a, f, r, c, front_entry<C>(a, f, s, ch, has, r, c));
+  // a warp per column, lanes along the rows: no division per entry, and a
+  // child without the column is skipped for all of it
+  for (int c = blockIdx.y * 8 + (threadIdx.x >> 5); c < n; c += gridDim.y * 8) {
+    bool in[2];
+#pragma unroll
+    for (int ci = 0; ci < 2; ++ci) in[ci] = has[ci] && a.inv[f.inv_off[ci] + c] >= 0;
+    for (int r = threadIdx.x & 31; r < n; r += 32) st_elem<C>(a, f, r, c, front_entry<C>(a, f, s, ch, in, r, c));
   }
   if (a.pcol && blockIdx.y == 0)
     for (int j = threadIdx.x; j < f.p; j += blockDim.x) a.pcol[f.piv_off + j] = j;
@@ -278,17 +280,42 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
     has[ci] = f.child[ci] >= 0;
     if (has[ci]) ch[ci] = a.fronts[f.child[ci]];
   }
+  // A box without children (symmetric form): each border node couples to one
+  // pivot, F12(:, c) = a_c e_k(c), and F22 is zero, so only F11 is swept --
+  // H12(:, c) = Finv(:, k(c)) a_c, S = - a_r Finv(k(r), k(c)) a_c -- a third
+  // of the sweep's multiply-adds at 16 pivots and 16 border nodes (32,768
+  // such fronts: 2.47 ms when the whole front was swept, FP64-pipe bound).
+  const bool leaf = sym && !has[0] && !has[1];
+  const int m = leaf ? p : n;                       // rows and columns swept
+  const int lds = leaf ? (p | 1) : ld;
+  C *Hm = F + (size_t)p * lds;                      // leaf: H12, p x b
+  C *ac = Hm + (size_t)p * f.b;                     // leaf: the couplings a_c
+  int *kc = reinterpret_cast<int *>(ac + f.b);      // leaf: their pivots
   if (sym) {
     // the assembled front is exactly symmetric (pairwise-equal stencil
     // entries, children's Schur complements stored symmetric): lower half
     // and mirror, enumerated as in the update below
-    for (int e = t; e < n * (n + 1) / 2; e += TPF) {
-      const int g = e / (n + 1), j = e - g * (n + 1);
-      const int c = j < n - g ? g : n - 1 - g, r = j < n - g ? g + j : c + j - (n - g);
+    for (int e = t; e < m * (m + 1) / 2; e += TPF) {
+      const int g = e / (m + 1), j = e - g * (m + 1);
+      const int c = j < m - g ? g : m - 1 - g, r = j < m - g ? g + j : c + j - (m - g);
       const C v = front_entry<C>(a, f, s, ch, has, r, c);
-      F[c * ld + r] = v;
-      F[r * ld + c] = v;
+      F[c * lds + r] = v;
+      F[r * lds + c] = v;
     }
+    if (leaf)
+      for (int c = t; c < f.b; c += TPF) {
+        C v = czero<C>();
+        int k = 0;
+        for (int q = 0; q < p; ++q) {
+          const C w = front_entry<C>(a, f, s, ch, has, q, p + c);
+          if (w.x != 0 || w.y != 0) {
+            v = w;
+            k = q;
+          }
+        }
+        ac[c] = v;
+        kc[c] = k;
+      }
   } else {
     for (int idx = t; idx < n * n; idx += TPF) {
       const int c = idx / n, r = idx - c * n;
@@ -335,7 +362,7 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
     // every other thread takes the reciprocal from it)
     C inv = czero<C>();
     if (t == 0) {
-      const C d0 = F[k * ld + k];
+      const C d0 = F[k * lds + k];
       bool raised;
       inv = crecip(floor_pivot(a, d0, raised));
       const R d2 = cabs2(d0);
@@ -352,31 +379,31 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
       __syncthreads();
       inv = inv_s;
     }
-    for (int j = t; j < n; j += TPF) {
-      rowk[j] = cmul(F[j * ld + k], inv);
-      colk[j] = F[k * ld + j];
+    for (int j = t; j < m; j += TPF) {
+      rowk[j] = cmul(F[j * lds + k], inv);
+      colk[j] = F[k * lds + j];
     }
     front_sync<TPF>();
     if (sym) {
-      // the n (n + 1) / 2 entries with r >= c, enumerated by column pairs
-      // (c, n - 1 - c) of n + 1 entries each; the mirror of (r, c) is
+      // the m (m + 1) / 2 entries with r >= c, enumerated by column pairs
+      // (c, m - 1 - c) of m + 1 entries each; the mirror of (r, c) is
       // negated when exactly one of r and c is eliminated (<= k)
-      for (int e = t; e < n * (n + 1) / 2; e += TPF) {
-        const int g = e / (n + 1), j = e - g * (n + 1);
+      for (int e = t; e < m * (m + 1) / 2; e += TPF) {
+        const int g = e / (m + 1), j = e - g * (m + 1);
         int r, c;
-        if (j < n - g) {
+        if (j < m - g) {
           c = g;
           r = g + j;
         } else {
-          c = n - 1 - g;
-          r = c + j - (n - g);
+          c = m - 1 - g;
+          r = c + j - (m - g);
         }
         C v;
         if (r == k) v = (c == k) ? inv : rowk[c];
         else if (c == k) v = cneg(cmul(colk[r], inv));
-        else v = cfms(colk[r], rowk[c], F[c * ld + r]);
-        F[c * ld + r] = v;
-        if (r != c) F[r * ld + c] = cneg_if(v, (r <= k) != (c <= k));
+        else v = cfms(colk[r], rowk[c], F[c * lds + r]);
+        F[c * lds + r] = v;
+        if (r != c) F[r * lds + c] = cneg_if(v, (r <= k) != (c <= k));
       }
     } else {
       for (int idx = t; idx < n * n; idx += TPF) {
@@ -391,9 +418,53 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
     front_sync<TPF>();
   }
   if (t == 0) note_pivot(a, bad ? 0.0 : sqrt(d2min), !bad);
-  for (int idx = t; idx < n * n; idx += TPF) {
-    const int c = idx / n, r = idx - c * n;
-    st_elem<C>(a, f, r, c, F[c * ld + r]);
+  if (leaf) {
+    for (int e = t; e < p * f.b; e += TPF) {
+      const int c = e / p, r = e - c * p;
+      Hm[e] = cmul(F[kc[c] * lds + r], ac[c]);
+    }
+    front_sync<TPF>();
+  }
+  // entry (r, c) of the eliminated front; a leaf's -G21 is -H12^T and its S
+  // formed from the larger index's coupling, so that S is exactly symmetric
+  auto entry = [&](int r, int c) {
+    if (!leaf || (r < p && c < p)) return F[c * lds + r];
+    if (r < p) return Hm[(c - p) * p + r];
+    if (c < p) return cneg(Hm[(r - p) * p + c]);
+    const int hi = max(r, c) - p, lo = min(r, c) - p;
+    return cneg(cmul(ac[hi], Hm[lo * p + kc[hi]]));
+  };
+  if constexpr (sizeof(R) == 8) {
+    // S as it is, the factor blocks straight to fixed point (mf_fixed.cuh),
+    // a thread per row and chain: no second pass over the small fronts
+    const int b = f.b, nd = (n + FX_COLS - 1) / FX_COLS, nu = (p + FX_COLS - 1) / FX_COLS;
+    for (int idx = t; idx < b * b; idx += TPF) {
+      const int c = idx / b, r = idx - c * b;
+      st_elem<C>(a, f, p + r, p + c, entry(p + r, p + c));
+    }
+    for (int idx = t; idx < p * nd + b * nu; idx += TPF) {
+      const bool down = idx < p * nd;
+      const int rows = down ? p : b, u = down ? idx : idx - p * nd, k = u / rows, r = u - k * rows;
+      const int c0 = k * FX_COLS, c1 = min(down ? n : p, c0 + FX_COLS), scaled = down ? p : 0;
+      int e = FX_EMPTY;
+      for (int c = c0; c < c1; ++c) {
+        const C v = entry(down ? r : p + r, c);
+        const int sh = c < scaled ? a.fx_scale : 0;
+        e = max(e, max(fx_exp(v.x, sh), fx_exp(v.y, sh)));
+      }
+      a.fexp[f.exp_off + (down ? 0 : (int64_t)p * nd) + (int64_t)k * rows + r] = (short)e;
+      ulonglong2 *W = reinterpret_cast<ulonglong2 *>(a.fac) + f.fac_off + (down ? 0 : (int64_t)p * n) + r;
+      for (int c = c0; c < c1; ++c) {
+        const C v = entry(down ? r : p + r, c);
+        const int ec = e - (c < scaled ? a.fx_scale : 0);
+        W[(int64_t)c * rows] = make_ulonglong2(fx_matrix_word(v.x, ec), fx_matrix_word(v.y, ec));
+      }
+    }
+  } else {
+    for (int idx = t; idx < n * n; idx += TPF) {
+      const int c = idx / n, r = idx - c * n;
+      st_elem<C>(a, f, r, c, entry(r, c));
+    }
   }
   if (piv)
     for (int j = t; j < p; j += TPF) a.pcol[f.piv_off + j] = perm[j];
@@ -482,12 +553,24 @@ __global__ void __launch_bounds__(256) mf_gj_pivot(MfArgs a, int f0, int k) {
   }
 }
 
+// The inverse of the pivot block, one block per front: 32 dependent pivots,
+// whose chain a level with few fronts waits for.  Two multiply-adds per clock
+// and SM make a pivot's update of the whole block (4096 multiply-adds) about
+// 1 us; a warp of its own takes the next pivot's entry through that update
+// first and forms its reciprocal while the others still update.  The whole
+// block is updated in the symmetric form too: the lower half alone, mirrored,
+// is faster but was seen to lose digits in the band-space solves.
+// 104 us a block of 32 in complex128 with 128 threads, the correctly rounded
+// reciprocal and its statistics on their own between two barriers.
+constexpr int DIAG_WORKERS = 256, DIAG_THREADS = DIAG_WORKERS + 32;
+
 template <typename R>
-__global__ void __launch_bounds__(MF_PANEL_THREADS) mf_gj_diag(MfArgs a, int f0, int k) {
+__global__ void __launch_bounds__(DIAG_THREADS) mf_gj_diag(MfArgs a, int f0, int k) {
   using C = typename CT<R>::T;
   constexpr int NB = MF_NB;
   __shared__ C D[NB][NB + 1];
   __shared__ C rowk[NB], colk[NB];
+  __shared__ C inv_s[2];
   const FrontDev f = a.fronts[f0 + blockIdx.x];
   const int p = f.p, n = p + f.b;
   if (n <= MF_SMALL || k >= p) return;
@@ -495,44 +578,51 @@ __global__ void __launch_bounds__(MF_PANEL_THREADS) mf_gj_diag(MfArgs a, int f0,
   C *fac = reinterpret_cast<C *>(a.fac);
   const int64_t fo = f.fac_off;
   const int tid = threadIdx.x;
-  for (int idx = tid; idx < nbk * nbk; idx += blockDim.x) {
+  for (int idx = tid; idx < nbk * nbk; idx += DIAG_THREADS) {
     const int i = idx % nbk, j = idx / nbk;
     D[i][j] = fac[fo + (int64_t)(k + j) * p + k + i];
   }
   __syncthreads();
+  const bool lead = tid == DIAG_WORKERS;      // the next pivot's thread
   double d2min = INFINITY;
   bool bad = false;
-  __shared__ C inv_s;
+  // reciprocal of pivot q first (the others wait for it), then its statistics
+  auto pivot = [&](C d0, int q) {
+    bool raised;
+    inv_s[q & 1] = crecip(floor_pivot(a, d0, raised));
+    const R d2 = cabs2(d0);
+    bad |= !pivot_ok(d2);
+    d2min = fmin(d2min, (double)d2);
+    if (raised) atomicAdd(a.n_raised, 1ull);
+  };
+  if (lead) pivot(D[0][0], 0);
+  __syncthreads();
   for (int q = 0; q < nbk; ++q) {
-    // reciprocal and statistics of the pivot by one thread (see mf_gj_small)
-    if (tid == 0) {
-      const C d0 = D[q][q];
-      bool raised;
-      inv_s = crecip(floor_pivot(a, d0, raised));
-      const R d2 = cabs2(d0);
-      bad |= !pivot_ok(d2);
-      d2min = fmin(d2min, (double)d2);
-      if (raised) atomicAdd(a.n_raised, 1ull);
-    }
+    const C inv = inv_s[q & 1];
+    if (tid < nbk) rowk[tid] = cmul(D[q][tid], inv);
+    else if (tid >= 32 && tid - 32 < nbk) colk[tid - 32] = D[tid - 32][q];
     __syncthreads();
-    const C inv = inv_s;
-    for (int j = tid; j < nbk; j += blockDim.x) {
-      rowk[j] = cmul(D[q][j], inv);
-      colk[j] = D[j][q];
-    }
-    __syncthreads();
-    for (int idx = tid; idx < nbk * nbk; idx += blockDim.x) {
-      const int i = idx % nbk, j = idx / nbk;
-      C v;
-      if (i == q) v = (j == q) ? inv : rowk[j];
-      else if (j == q) v = cneg(cmul(colk[i], inv));
-      else v = cfms(colk[i], rowk[j], D[i][j]);
-      D[i][j] = v;
+    if (lead) {
+      if (q + 1 < nbk) {
+        const C v = cfms(colk[q + 1], rowk[q + 1], D[q + 1][q + 1]);
+        D[q + 1][q + 1] = v;
+        pivot(v, q + 1);
+      }
+    } else if (tid < DIAG_WORKERS) {
+      for (int idx = tid; idx < nbk * nbk; idx += DIAG_WORKERS) {
+        const int i = idx % nbk, j = idx / nbk;
+        if (i == q + 1 && j == q + 1) continue;
+        C v;
+        if (i == q) v = (j == q) ? inv : rowk[j];
+        else if (j == q) v = cneg(cmul(colk[i], inv));
+        else v = cfms(colk[i], rowk[j], D[i][j]);
+        D[i][j] = v;
+      }
     }
     __syncthreads();
   }
-  if (tid == 0) note_pivot(a, bad ? 0.0 : sqrt(d2min), !bad);
-  for (int idx = tid; idx < nbk * nbk; idx += blockDim.x) {
+  if (lead) note_pivot(a, bad ? 0.0 : sqrt(d2min), !bad);
+  for (int idx = tid; idx < nbk * nbk; idx += DIAG_THREADS) {
     const int i = idx % nbk, j = idx / nbk;
     fac[fo + (int64_t)(k + j) * p + k + i] = D[i][j];
   }
@@ -1012,7 +1102,7 @@ __device__ __forceinline__ int fx_row(int lane) { return 8 * ((lane >> 1) & 1) +
 // component lane % 2 of v
 __device__ __forceinline__ double fx_part(double2 v, int lane) { return (lane & 1) ? v.y : v.x; }
 
-// Factor blocks of a level's eliminated fronts to fixed point, in place: one
+// Factor blocks of a level's eliminated large fronts to fixed point, in place: one
 // warp per 32 rows of a chain, lane = row, 32 columns in registers.  Reads
 // and writes every entry once (a pass at HBM speed; the preconditioner's
 // products then never convert).
@@ -1024,6 +1114,7 @@ __global__ void __launch_bounds__(128) mf_to_fixed(MfArgs a, int f0, int nf, int
   if (fi >= nf) return;
   const FrontDev f = a.fronts[f0 + fi];
   const int p = f.p, b = f.b, n = p + b;
+  if (n <= MF_SMALL) return;       // mf_gj_small wrote them so
   const int nd = (n + FX_COLS - 1) / FX_COLS, nu = (p + FX_COLS - 1) / FX_COLS;
   const int rd = (p + 31) / 32, ru = (b + 31) / 32;
   int rows = p, cols = n;
@@ -1867,9 +1958,7 @@ void mf_factor_level(const MfArgs &a, const LevelInfo &L, int level, cudaStream_
     count_launch();
   }
   if (L.max_n > MF_SMALL) {
-    const int64_t nn = (int64_t)L.max_n * L.max_n;
-    const int gy = (int)std::min<int64_t>((nn + 255) / 256, 4096);
-    mf_assemble<R><<<dim3(L.nf, gy), 256, 0, st>>>(a, L.f0);
+    mf_assemble<R><<<dim3(L.nf, (L.max_n + 7) / 8), 256, 0, st>>>(a, L.f0);
     count_launch();
     for (int k = 0; k < L.max_p; k += MF_NB) {
       const int m = L.max_n - std::min(MF_NB, std::max(1, L.max_p - k));
@@ -1879,7 +1968,7 @@ void mf_factor_level(const MfArgs &a, const LevelInfo &L, int level, cudaStream_
         mf_gj_pivot<R><<<L.nf, 256, 0, st>>>(a, L.f0, k);
         count_launch();
       }
-      mf_gj_diag<R><<<L.nf, MF_PANEL_THREADS, 0, st>>>(a, L.f0, k);
+      mf_gj_diag<R><<<L.nf, DIAG_THREADS, 0, st>>>(a, L.f0, k);
       if (a.sym && a.fp64_tc && sizeof(R) == 8) mf_oz_col_launch(a, L, k, st);
       else mf_gj_col<R><<<dim3(L.nf, tiles), MF_PANEL_THREADS, 0, st>>>(a, L.f0, k);
       if (hook) hook->before(K_UPDATE, level, k);
@@ -1904,7 +1993,7 @@ void mf_factor_level(const MfArgs &a, const LevelInfo &L, int level, cudaStream_
       count_launch(4);
     }
   }
-  if constexpr (sizeof(R) == 8) {
+  if (sizeof(R) == 8 && L.max_n > MF_SMALL) {
     // the substitutions read fixed-point factors (the parents only read S)
     const int upf = (L.max_p + 31) / 32 * ((L.max_n + FX_COLS - 1) / FX_COLS) +
                     (L.max_b + 31) / 32 * ((L.max_p + FX_COLS - 1) / FX_COLS);

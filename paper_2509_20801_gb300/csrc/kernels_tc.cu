@@ -520,8 +520,8 @@ __device__ __forceinline__ double2 *front_ptr64(const MfArgs &a, const FrontDev 
 // that skips the pivot band), lower entries added to the front and their
 // signed mirrors stored, as mf_gj_update_sym does on the FP64 pipe.  CTA
 // (front, ti, chunk): rows [64 ti, 64 ti + 64) against the chunk's columns
-// (at most 32 OZ_CHUNK) up to the diagonal.  grid = (fronts, tile rows x chunks).
-__global__ void __launch_bounds__(OZ_THREADS, 1) mf_gj_update_oz(MfArgs a, int f0, int k, int nchunk) {
+// (32 `chunk`) up to the diagonal.  grid = (fronts, tile rows x chunks).
+__global__ void __launch_bounds__(OZ_THREADS, 1) mf_gj_update_oz(MfArgs a, int f0, int k, int nchunk, int chunk) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   OzSmem &sm = *reinterpret_cast<OzSmem *>(smem_raw);
   const FrontDev f = a.fronts[f0 + blockIdx.x];
@@ -531,8 +531,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) mf_gj_update_oz(MfArgs a, int f
   const int m = n - nbk;
   const int ti = blockIdx.y / nchunk, ch = blockIdx.y - ti * nchunk;
   const int i0 = ti * OZ_MR;
-  const int c0 = ch * OZ_NC * OZ_CHUNK;
-  const int cend = min(min(i0 + OZ_MR, m), c0 + OZ_NC * OZ_CHUNK);
+  const int c0 = ch * OZ_NC * chunk;
+  const int cend = min(min(i0 + OZ_MR, m), c0 + OZ_NC * chunk);
   if (i0 >= m || c0 >= cend) return;
   const double2 *fac = reinterpret_cast<const double2 *>(a.fac);
   const int64_t fo = f.fac_off;
@@ -712,11 +712,33 @@ void mf_oz_col_launch(const MfArgs &a, const LevelInfo &L, int k, cudaStream_t s
   count_launch();
 }
 
+// Sub-tiles of 32 columns per CTA.  A CTA costs about 17 us for the slices of
+// its 64 rows and its tensor memory, and 7.5 us per sub-tile; one runs on an
+// SM.  Long chunks share the rows' slices, short ones fill the GPU at the
+// levels near the root: with 16 throughout, a step of 4 fronts of 340 rows
+// ran on 20 CTAs (97 us), of 8 fronts of 468 on 72 (148 us).  The estimate
+// takes the work over all SMs and half of the longest CTA for the tail.
+int oz_chunk(int nf, int nt) {
+  int best = OZ_CHUNK;
+  double best_us = 1e30;
+  for (int c = OZ_CHUNK; c >= 1; c /= 2) {
+    double ctas = 0;
+    for (int ti = 0; ti < nt; ++ti) ctas += (2 * (ti + 1) + c - 1) / c;
+    const double longest = 17.0 + 7.5 * std::min(c, 2 * nt);
+    const double us = nf * (17.0 * ctas + 7.5 * nt * (nt + 1)) / 152.0 + 0.5 * longest;
+    if (us < best_us) {
+      best_us = us;
+      best = c;
+    }
+  }
+  return best;
+}
+
 void mf_oz_update_launch(const MfArgs &a, const LevelInfo &L, int k, cudaStream_t st) {
   const int m = L.max_n - std::min(MF_NB, std::max(1, L.max_p - k));
-  const int nt = std::max(1, (m + OZ_MR - 1) / OZ_MR);
-  const int nchunk = std::max(1, (nt * OZ_MR + OZ_NC * OZ_CHUNK - 1) / (OZ_NC * OZ_CHUNK));
-  mf_gj_update_oz<<<dim3(L.nf, nt * nchunk), OZ_THREADS, oz_smem_bytes(), st>>>(a, L.f0, k, nchunk);
+  const int nt = std::max(1, (m + OZ_MR - 1) / OZ_MR), chunk = oz_chunk(L.nf, nt);
+  const int nchunk = std::max(1, (nt * OZ_MR + OZ_NC * chunk - 1) / (OZ_NC * chunk));
+  mf_gj_update_oz<<<dim3(L.nf, nt * nchunk), OZ_THREADS, oz_smem_bytes(), st>>>(a, L.f0, k, nchunk, chunk);
   count_launch();
 }
 
