@@ -118,6 +118,10 @@ __device__ __forceinline__ int unband(int i, int k, int nbk) { return i < k ? i 
 // is a pivot here (Eq. 2 with the stretched couplings of Eq. 9, strip-local
 // x couplings), plus the children's Schur complements placed by the inverse
 // extend-add maps.
+// whether a product with both stretches changes anything: 1 + i sigma each,
+// exactly 1 outside the PMLs (the FP64 pipe has better to do there)
+__device__ __forceinline__ bool stretched(double2 s, double2 t) { return s.y != 0.0 || t.y != 0.0; }
+
 template <typename C>
 __device__ __forceinline__ C front_entry(const MfArgs &a, const FrontDev &f, const StripDev &s, const FrontDev *ch,
                                          const bool *has, int r, int c) {
@@ -138,13 +142,15 @@ __device__ __forceinline__ C front_entry(const MfArgs &a, const FrontDev &f, con
         double2 d0;
         d0.x = a.k0sq * a.eps[(int64_t)(s.x0 + ux) * a.H + s.y0 + uy] - xm.x - xp.x - ym.x - yp.x;
         d0.y = -xm.y - xp.y - ym.y - yp.y;
-        v = cmul(cmul(sxu, syu), d0);
+        v = stretched(sxu, syu) ? cmul(cmul(sxu, syu), d0) : d0;
       } else if (d == -H || d == H) {
         const int lx = d == -H ? ux - 1 : ux;     // the pair's left column
-        v = cmul(cmul(a.lsx[s.coef_off + lx], a.cxp[s.coef_off + lx]), syu);
+        const double2 sl = a.lsx[s.coef_off + lx], cp = a.cxp[s.coef_off + lx];
+        v = stretched(sl, syu) ? cmul(cmul(sl, cp), syu) : cp;
       } else if ((d == -1 && uy > 0) || (d == 1 && uy < H - 1)) {
         const int ly = d == -1 ? uy - 1 : uy;     // the pair's lower row
-        v = cmul(cmul(a.lsy[s.ycoef_off + ly], a.cyp[s.ycoef_off + ly]), sxu);
+        const double2 sl = a.lsy[s.ycoef_off + ly], cp = a.cyp[s.ycoef_off + ly];
+        v = stretched(sl, sxu) ? cmul(cmul(sl, cp), sxu) : cp;
       }
     } else if (d == 0) {
       const double2 xm = a.cxm[s.coef_off + ux], xp = a.cxp[s.coef_off + ux];
@@ -199,6 +205,15 @@ __global__ void __launch_bounds__(256) mf_assemble(MfArgs a, int f0) {
   }
   if (a.pcol && blockIdx.y == 0)
     for (int j = threadIdx.x; j < f.p; j += blockDim.x) a.pcol[f.piv_off + j] = j;
+}
+
+// Entry (r, c) after pivot k of a Gauss-Jordan sweep: row = the scaled pivot
+// row's entry in column c, with the pivot's reciprocal in column k; col = the
+// pivot column's entry in row r; old = the entry before.  One multiply-add
+// for all, so that lanes on the pivot column take no branch of their own.
+template <typename C> __device__ __forceinline__ C swept_entry(bool on_row, bool on_col, C col, C row, C old) {
+  const C v = cfms(col, row, on_col ? czero<C>() : old);
+  return on_row ? row : v;
 }
 
 // ------------------------------------------------ small fronts, in smem
@@ -304,15 +319,14 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
     }
     if (leaf)
       for (int c = t; c < f.b; c += TPF) {
-        C v = czero<C>();
+        // the pivot next to border node w: the same row or the same column
+        const int H = s.y1 - s.y0, w = a.nodes[f.node_off + p + c];
         int k = 0;
         for (int q = 0; q < p; ++q) {
-          const C w = front_entry<C>(a, f, s, ch, has, q, p + c);
-          if (w.x != 0 || w.y != 0) {
-            v = w;
-            k = q;
-          }
+          const int u = a.nodes[f.node_off + q], d = w - u;
+          if (d == H || d == -H || ((d == 1 || d == -1) && u / H == w / H)) k = q;
         }
+        const C v = front_entry<C>(a, f, s, ch, has, k, p + c);
         ac[c] = v;
         kc[c] = k;
       }
@@ -380,7 +394,7 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
       inv = inv_s;
     }
     for (int j = t; j < m; j += TPF) {
-      rowk[j] = cmul(F[j * lds + k], inv);
+      rowk[j] = j == k ? inv : cmul(F[j * lds + k], inv);
       colk[j] = F[k * lds + j];
     }
     front_sync<TPF>();
@@ -398,21 +412,14 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
           c = m - 1 - g;
           r = c + j - (m - g);
         }
-        C v;
-        if (r == k) v = (c == k) ? inv : rowk[c];
-        else if (c == k) v = cneg(cmul(colk[r], inv));
-        else v = cfms(colk[r], rowk[c], F[c * lds + r]);
+        const C v = swept_entry(r == k, c == k, colk[r], rowk[c], F[c * lds + r]);
         F[c * lds + r] = v;
         if (r != c) F[r * lds + c] = cneg_if(v, (r <= k) != (c <= k));
       }
     } else {
       for (int idx = t; idx < n * n; idx += TPF) {
         const int c = idx / n, r = idx - c * n;
-        C v;
-        if (r == k) v = (c == k) ? inv : rowk[c];
-        else if (c == k) v = cneg(cmul(colk[r], inv));
-        else v = cfms(colk[r], rowk[c], F[c * ld + r]);
-        F[c * ld + r] = v;
+        F[c * ld + r] = swept_entry(r == k, c == k, colk[r], rowk[c], F[c * ld + r]);
       }
     }
     front_sync<TPF>();
@@ -553,25 +560,75 @@ __global__ void __launch_bounds__(256) mf_gj_pivot(MfArgs a, int f0, int k) {
   }
 }
 
+// Symmetric form: the pivot rows after step k without the row product.
+// The working matrix after the step is symmetric within the eliminated and
+// within the remaining indices and antisymmetric between them, so pivot row
+// k + i at column c is the column just written by mf_gj_col at (c, k + i),
+// negated when c is not yet eliminated (c >= k + nbk) and kept when c < k.
+// A transpose through shared memory: reads along c, writes along i.  One
+// block of THREADS threads, MIRROR_COLS columns.
+constexpr int MIRROR_COLS = 64;
+
+template <typename R, int THREADS>
+__device__ __forceinline__ void mirror_rows(const MfArgs &a, const FrontDev &f, int k, int tile,
+                                            typename CT<R>::T (*T)[MF_NB + 1]) {
+  using C = typename CT<R>::T;
+  const int p = f.p, n = p + f.b;
+  if (n <= MF_SMALL || k < 0 || k >= p) return;
+  const int nbk = min(MF_NB, p - k);
+  const int cbase = tile * MIRROR_COLS, cols = n - nbk;
+  if (cbase >= cols) return;
+  C *fac = reinterpret_cast<C *>(a.fac);
+  const int64_t fo = f.fac_off;
+  const int ncol = min(MIRROR_COLS, cols - cbase);
+  for (int idx = threadIdx.x; idx < nbk * MIRROR_COLS; idx += THREADS) {
+    const int cc = idx % MIRROR_COLS, i = idx / MIRROR_COLS;
+    if (cc >= ncol) continue;
+    const int c = unband(cbase + cc, k, nbk);
+    T[cc][i] = cneg_if(ld_elem<C>(a, f, c, k + i), c >= k);
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < MF_NB * ncol; idx += THREADS) {
+    const int i = idx % MF_NB, cc = idx / MF_NB;
+    if (i < nbk) fac[fo + (int64_t)unband(cbase + cc, k, nbk) * p + k + i] = T[cc][i];
+  }
+}
+
+// after the last step of a level
+template <typename R>
+__global__ void __launch_bounds__(MF_PANEL_THREADS) mf_gj_row_mirror(MfArgs a, int f0, int k) {
+  __shared__ typename CT<R>::T T[MIRROR_COLS][MF_NB + 1];
+  mirror_rows<R, MF_PANEL_THREADS>(a, a.fronts[f0 + blockIdx.x], k, blockIdx.y, T);
+}
+
 // The inverse of the pivot block, one block per front: 32 dependent pivots,
 // whose chain a level with few fronts waits for.  Two multiply-adds per clock
-// and SM make a pivot's update of the whole block (4096 multiply-adds) about
-// 1 us; a warp of its own takes the next pivot's entry through that update
-// first and forms its reciprocal while the others still update.  The whole
-// block is updated in the symmetric form too: the lower half alone, mirrored,
-// is faster but was seen to lose digits in the band-space solves.
-// 104 us a block of 32 in complex128 with 128 threads, the correctly rounded
-// reciprocal and its statistics on their own between two barriers.
+// and SM make a pivot's update of the block (4096 multiply-adds) about 1 us; a
+// warp of its own takes the next pivot through the update and forms its
+// reciprocal while the others still update.  (One triangle, mirrored in the
+// symmetric form, takes no less: its rows end within warps.)
+// 104 us a block of 32 in complex128 with 128 threads, the pivot row and
+// column on branches of their own -- the FP64 pipe pays a branch that one lane
+// takes like all -- and the correctly rounded reciprocal and its statistics
+// between two barriers.
+// The blocks past the first of a front (symmetric form) mirror the previous
+// step's pivot rows: the column panel of this step needs both, and mirroring
+// takes a fraction of the inverse's time (23 us as a launch of its own).
 constexpr int DIAG_WORKERS = 256, DIAG_THREADS = DIAG_WORKERS + 32;
 
 template <typename R>
 __global__ void __launch_bounds__(DIAG_THREADS) mf_gj_diag(MfArgs a, int f0, int k) {
   using C = typename CT<R>::T;
   constexpr int NB = MF_NB;
-  __shared__ C D[NB][NB + 1];
+  __shared__ C T[MIRROR_COLS][NB + 1];
+  const FrontDev f = a.fronts[f0 + blockIdx.x];
+  if (blockIdx.y > 0) {
+    mirror_rows<R, DIAG_THREADS>(a, f, k - NB, blockIdx.y - 1, T);
+    return;
+  }
+  C(*D)[NB + 1] = T;
   __shared__ C rowk[NB], colk[NB];
   __shared__ C inv_s[2];
-  const FrontDev f = a.fronts[f0 + blockIdx.x];
   const int p = f.p, n = p + f.b;
   if (n <= MF_SMALL || k >= p) return;
   const int nbk = min(NB, p - k);
@@ -583,45 +640,42 @@ __global__ void __launch_bounds__(DIAG_THREADS) mf_gj_diag(MfArgs a, int f0, int
     D[i][j] = fac[fo + (int64_t)(k + j) * p + k + i];
   }
   __syncthreads();
-  const bool lead = tid == DIAG_WORKERS;      // the next pivot's thread
-  double d2min = INFINITY;
-  bool bad = false;
-  // reciprocal of pivot q first (the others wait for it), then its statistics
-  auto pivot = [&](C d0, int q) {
-    bool raised;
-    inv_s[q & 1] = crecip(floor_pivot(a, d0, raised));
-    const R d2 = cabs2(d0);
-    bad |= !pivot_ok(d2);
-    d2min = fmin(d2min, (double)d2);
-    if (raised) atomicAdd(a.n_raised, 1ull);
-  };
-  if (lead) pivot(D[0][0], 0);
-  __syncthreads();
-  for (int q = 0; q < nbk; ++q) {
-    const C inv = inv_s[q & 1];
-    if (tid < nbk) rowk[tid] = cmul(D[q][tid], inv);
-    else if (tid >= 32 && tid - 32 < nbk) colk[tid - 32] = D[tid - 32][q];
-    __syncthreads();
-    if (lead) {
-      if (q + 1 < nbk) {
-        const C v = cfms(colk[q + 1], rowk[q + 1], D[q + 1][q + 1]);
-        D[q + 1][q + 1] = v;
-        pivot(v, q + 1);
-      }
-    } else if (tid < DIAG_WORKERS) {
+  if (tid >= DIAG_WORKERS) {
+    // the pivots' warp (all lanes alike): pivot q + 1 from the block as step
+    // q - 1 left it, with the update's own arithmetic
+    C d0 = D[0][0];
+    double d2min = INFINITY;
+    bool bad = false;
+    for (int q = 0; q < nbk; ++q) {
+      bool raised;
+      const C inv = crecip(floor_pivot(a, d0, raised));
+      if (tid == DIAG_WORKERS) inv_s[q & 1] = inv;
+      __syncthreads();                            // step q - 1 done, inv known
+      const int s = min(q + 1, nbk - 1);
+      const C col = D[s][q], row = D[q][s], dia = D[s][s];
+      __threadfence_block();
+      asm volatile("bar.arrive 1, %0;\n" ::"n"(DIAG_THREADS) : "memory");   // read before the workers write
+      const R d2 = cabs2(d0);
+      bad |= !pivot_ok(d2);
+      d2min = fmin(d2min, (double)d2);
+      if (raised && tid == DIAG_WORKERS) atomicAdd(a.n_raised, 1ull);
+      d0 = cfms(col, cmul(row, inv), dia);
+    }
+    if (tid == DIAG_WORKERS) note_pivot(a, bad ? 0.0 : sqrt(d2min), !bad);
+  } else {
+    for (int q = 0; q < nbk; ++q) {
+      __syncthreads();
+      const C inv = inv_s[q & 1];
+      if (tid < nbk) rowk[tid] = tid == q ? inv : cmul(D[q][tid], inv);
+      else if (tid >= 32 && tid - 32 < nbk) colk[tid - 32] = D[tid - 32][q];
+      asm volatile("bar.sync 1, %0;\n" ::"n"(DIAG_THREADS) : "memory");
       for (int idx = tid; idx < nbk * nbk; idx += DIAG_WORKERS) {
         const int i = idx % nbk, j = idx / nbk;
-        if (i == q + 1 && j == q + 1) continue;
-        C v;
-        if (i == q) v = (j == q) ? inv : rowk[j];
-        else if (j == q) v = cneg(cmul(colk[i], inv));
-        else v = cfms(colk[i], rowk[j], D[i][j]);
-        D[i][j] = v;
+        D[i][j] = swept_entry(i == q, j == q, colk[i], rowk[j], D[i][j]);
       }
     }
-    __syncthreads();
   }
-  if (lead) note_pivot(a, bad ? 0.0 : sqrt(d2min), !bad);
+  __syncthreads();
   for (int idx = tid; idx < nbk * nbk; idx += DIAG_THREADS) {
     const int i = idx % nbk, j = idx / nbk;
     fac[fo + (int64_t)(k + j) * p + k + i] = D[i][j];
@@ -713,43 +767,6 @@ __global__ void __launch_bounds__(MF_PANEL_THREADS) mf_gj_row(MfArgs a, int f0, 
   for (int idx = tid; idx < nbk * ncol; idx += blockDim.x) {
     const int i = idx % nbk, cc = idx / nbk;
     fac[fo + (int64_t)unband(cbase + cc, k, nbk) * p + k + i] = T[cc][i];
-  }
-}
-
-// Symmetric form: the pivot rows after step k without the row product.
-// The working matrix after the step is symmetric within the eliminated and
-// within the remaining indices and antisymmetric between them, so pivot row
-// k + i at column c is the column just written by mf_gj_col at (c, k + i),
-// negated when c is not yet eliminated (c >= k + nbk) and kept when c < k.
-// A transpose through shared memory: reads along c, writes along i.
-template <typename R>
-__global__ void __launch_bounds__(MF_PANEL_THREADS) mf_gj_row_mirror(MfArgs a, int f0, int k) {
-  using C = typename CT<R>::T;
-  constexpr int NB = MF_NB, TILE = MF_PANEL_THREADS, HALF = TILE / 2;
-  __shared__ C T[HALF][NB + 1];
-  const FrontDev f = a.fronts[f0 + blockIdx.x];
-  const int p = f.p, n = p + f.b;
-  if (n <= MF_SMALL || k >= p) return;
-  const int nbk = min(NB, p - k);
-  const int cols = n - nbk;
-  C *fac = reinterpret_cast<C *>(a.fac);
-  const int64_t fo = f.fac_off;
-  const int tid = threadIdx.x;
-  for (int h = 0; h < 2; ++h) {       // the block's TILE columns, HALF at a time
-    const int cbase = blockIdx.y * TILE + h * HALF;
-    if (cbase >= cols) return;
-    const int ncol = min(HALF, cols - cbase);
-    if (h) __syncthreads();
-    for (int idx = tid; idx < nbk * ncol; idx += TILE) {
-      const int cc = idx % ncol, i = idx / ncol, c = unband(cbase + cc, k, nbk);
-      const C v = ld_elem<C>(a, f, c, k + i);
-      T[cc][i] = cneg_if(v, c >= k);
-    }
-    __syncthreads();
-    for (int idx = tid; idx < nbk * ncol; idx += TILE) {
-      const int i = idx % nbk, cc = idx / nbk;
-      fac[fo + (int64_t)unband(cbase + cc, k, nbk) * p + k + i] = T[cc][i];
-    }
   }
 }
 
@@ -1154,14 +1171,6 @@ __global__ void __launch_bounds__(128) mf_to_fixed(MfArgs a, int f0, int nf, int
     }
 }
 
-// The sweeps' launches of consecutive levels overlap (programmatic dependent
-// launch): a block starts while the previous level's last ones still run,
-// loads what the factorization left (items, records, the first matrix
-// entries) and waits for that level's vectors here.  Without the launch
-// attribute both are no-ops.
-__device__ __forceinline__ void level_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-__device__ __forceinline__ void level_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-
 // Going up, part 1: one warp per front forms w = [t at the pivots; 0] plus
 // the children's update vectors (inverse extend-add maps); w_p goes to the
 // pivot slots of wloc (kept for the way down) and w_b is the initial value
@@ -1241,7 +1250,7 @@ __device__ __forceinline__ C wsrc_pivot(const MfArgs &a, const WSrc<C> &s, int k
     const int ux = node / s.Hl, uy = node - ux * s.Hl;
     const double2 sx = a.lsx[s.coef_off + ux], sy = a.lsy[s.ycoef_off + uy];
     // outside the PMLs both stretches are exactly 1
-    if (sx.y != 0.0 || sy.y != 0.0) w = cmul(w, to_c(cmul(sx, sy), C()));
+    if (stretched(sx, sy)) w = cmul(w, to_c(cmul(sx, sy), C()));
   }
   return wsrc_children(s, k, q, w);
 }
@@ -1779,28 +1788,12 @@ __global__ void __launch_bounds__(256) mf_seg_reduce(MfArgs a, const int2 *__res
   else reinterpret_cast<C *>(a.tloc)[a.strips[f.strip].vec_off + a.nodes[f.node_off + r]] = total;
 }
 
-// 256-thread blocks that may start before the stream's previous kernel ends
-// (the kernel calls level_wait before it reads what that one writes)
-template <typename... P, typename... A>
-void launch_overlapped(void (*kernel)(P...), dim3 grid, cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(256);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);   // errors: cudaGetLastError by the caller
-}
-
 template <typename R, bool UP, bool FUSED = false>
 void mf_seg_launch(const MfArgs &a, const int2 *items, int nitems, int cols_max, int64_t ldt, cudaStream_t st) {
   const int nsubmax = (cols_max + MF_SUB - 1) / MF_SUB;
   const int64_t units = (int64_t)nitems * nsubmax;
-  launch_overlapped(mf_seg_partial<R, UP, FUSED>, (unsigned)((units + 7) / 8), st, a, items, nitems, nsubmax, ldt);
-  launch_overlapped(mf_seg_reduce<R, UP, FUSED>, (unsigned)(((int64_t)nitems * 32 + 255) / 256), st, a, items,
+  launch_overlapped(mf_seg_partial<R, UP, FUSED>, (unsigned)((units + 7) / 8), 256, 0, st, a, items, nitems, nsubmax, ldt);
+  launch_overlapped(mf_seg_reduce<R, UP, FUSED>, (unsigned)(((int64_t)nitems * 32 + 255) / 256), 256, 0, st, a, items,
                     nitems, nsubmax);
   count_launch(2);
 }
@@ -1968,29 +1961,42 @@ void mf_factor_level(const MfArgs &a, const LevelInfo &L, int level, cudaStream_
         mf_gj_pivot<R><<<L.nf, 256, 0, st>>>(a, L.f0, k);
         count_launch();
       }
-      mf_gj_diag<R><<<L.nf, DIAG_THREADS, 0, st>>>(a, L.f0, k);
-      if (a.sym && a.fp64_tc && sizeof(R) == 8) mf_oz_col_launch(a, L, k, st);
-      else mf_gj_col<R><<<dim3(L.nf, tiles), MF_PANEL_THREADS, 0, st>>>(a, L.f0, k);
+      const int mirrors = (L.max_n + MIRROR_COLS - 1) / MIRROR_COLS;
+      mf_gj_diag<R><<<dim3(L.nf, a.sym && k > 0 ? 1 + mirrors : 1), DIAG_THREADS, 0, st>>>(a, L.f0, k);
+      count_launch();
+      if (a.sym && a.fp64_tc && sizeof(R) == 8) {
+        mf_oz_col_launch(a, L, k, st);
+      } else {
+        mf_gj_col<R><<<dim3(L.nf, tiles), MF_PANEL_THREADS, 0, st>>>(a, L.f0, k);
+        count_launch();
+      }
       if (hook) hook->before(K_UPDATE, level, k);
       if (tc_fmt >= 0 && sizeof(R) == 4) {
         mf_tc_update_launch(a, L, k, tc_fmt, st);
       } else if (a.sym && a.fp64_tc && sizeof(R) == 8) {
         mf_oz_update_launch(a, L, k, st);
-      } else if (a.sym) {
-        const int tm = L.upd_tile == 32 ? 32 : 64, nts = std::max(1, (m + tm - 1) / tm);
-        const size_t sm = sizeof(typename CT<R>::T) * (tm * (MF_NB + 1) + MF_NB * (tm + 1));
-        if (tm == 32) mf_gj_update_sym<R, 32><<<dim3(L.nf, nts * (nts + 1) / 2), 64, sm, st>>>(a, L.f0, k);
-        else mf_gj_update_sym<R, 64><<<dim3(L.nf, nts * (nts + 1) / 2), 256, sm, st>>>(a, L.f0, k);
-      } else if (L.upd_tile == 32) {
-        const int nt32 = std::max(1, (m + 31) / 32);
-        mf_gj_update32<R><<<dim3(L.nf, nt32 * nt32), 64, 0, st>>>(a, L.f0, k);
       } else {
-        mf_gj_update<R><<<dim3(L.nf, nt * nt), 256, gemm_smem<R>(), st>>>(a, L.f0, k);
+        if (a.sym) {
+          const int tm = L.upd_tile == 32 ? 32 : 64, nts = std::max(1, (m + tm - 1) / tm);
+          const size_t sm = sizeof(typename CT<R>::T) * (tm * (MF_NB + 1) + MF_NB * (tm + 1));
+          if (tm == 32) mf_gj_update_sym<R, 32><<<dim3(L.nf, nts * (nts + 1) / 2), 64, sm, st>>>(a, L.f0, k);
+          else mf_gj_update_sym<R, 64><<<dim3(L.nf, nts * (nts + 1) / 2), 256, sm, st>>>(a, L.f0, k);
+        } else if (L.upd_tile == 32) {
+          const int nt32 = std::max(1, (m + 31) / 32);
+          mf_gj_update32<R><<<dim3(L.nf, nt32 * nt32), 64, 0, st>>>(a, L.f0, k);
+        } else {
+          mf_gj_update<R><<<dim3(L.nf, nt * nt), 256, gemm_smem<R>(), st>>>(a, L.f0, k);
+        }
+        count_launch();
       }
       if (hook) hook->after(K_UPDATE, level, k);
-      if (a.sym) mf_gj_row_mirror<R><<<dim3(L.nf, tiles), MF_PANEL_THREADS, 0, st>>>(a, L.f0, k);
-      else mf_gj_row<R><<<dim3(L.nf, tiles), MF_PANEL_THREADS, row_smem<R>(), st>>>(a, L.f0, k);
-      count_launch(4);
+      if (!a.sym) {
+        mf_gj_row<R><<<dim3(L.nf, tiles), MF_PANEL_THREADS, row_smem<R>(), st>>>(a, L.f0, k);
+        count_launch();
+      } else if (k + MF_NB >= L.max_p) {   // other steps' rows: with the next step's pivot blocks
+        mf_gj_row_mirror<R><<<dim3(L.nf, mirrors), MF_PANEL_THREADS, 0, st>>>(a, L.f0, k);
+        count_launch();
+      }
     }
   }
   if (sizeof(R) == 8 && L.max_n > MF_SMALL) {
@@ -2038,8 +2044,8 @@ void mf_up_level(const MfArgs &a, const int2 *items, int nitems, int rows, int s
   const dim3 grid = rhs_grid((nitems + ipc - 1) / ipc, nrhs, nr);
 #define STDD_UP(RW, NRV)                                                                \
   do {                                                                                  \
-    if (fused) launch_overlapped(mf_up<R, RW, NRV, true>, grid, st, a, items, nitems, split, nrhs, ldt);  \
-    else launch_overlapped(mf_up<R, RW, NRV, false>, grid, st, a, items, nitems, split, nrhs, ldt);       \
+    if (fused) launch_overlapped(mf_up<R, RW, NRV, true>, grid, 256, 0, st, a, items, nitems, split, nrhs, ldt);  \
+    else launch_overlapped(mf_up<R, RW, NRV, false>, grid, 256, 0, st, a, items, nitems, split, nrhs, ldt);       \
   } while (0)
   if (rows == 16) {
     if (nr == 4) STDD_UP(16, MAXR); else if (nr == 2) STDD_UP(16, 2); else STDD_UP(16, 1);
@@ -2067,7 +2073,7 @@ void mf_down_level(const MfArgs &a, const int2 *items, int nitems, int rows, int
     while (!mf_split_fits(2 * sizeof(R), rows, split, cols_max, nr)) split /= 2;
   const int ipc = block_items<R>(rows) / split;
   const dim3 grid = rhs_grid((nitems + ipc - 1) / ipc, nrhs, nr);
-#define STDD_DOWN(RW, NRV) launch_overlapped(mf_down<R, RW, NRV>, grid, st, a, items, nitems, split, nrhs, ldt)
+#define STDD_DOWN(RW, NRV) launch_overlapped(mf_down<R, RW, NRV>, grid, 256, 0, st, a, items, nitems, split, nrhs, ldt)
   if (rows == 16) {
     if (nr == 4) STDD_DOWN(16, MAXR); else if (nr == 2) STDD_DOWN(16, 2); else STDD_DOWN(16, 1);
   } else {
