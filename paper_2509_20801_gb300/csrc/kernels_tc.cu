@@ -241,9 +241,12 @@ constexpr int OZ_ABYTES = 128 * 64 * 2;      // one A slice: 128 real rows x 64 
 constexpr int OZ_BBYTES = OZ_NC * 64 * 2;    // one B slice: 32 columns x 64 real K, BF16
 constexpr uint32_t OZ_TMEM_COLS = 512;       // 2 buffers x 8 accumulators x 32 columns
 constexpr int OZ_EMPTY = -2000;              // exponent of an all-zero row or column
-constexpr int OZ_WORKERS = 256;              // 8 warps stage and read out (w and w + 4: TMEM lanes 32 (w % 4))
+// 16 warps stage and read out (TMEM lanes 32 (w % 4)): slicing and reading out
+// are some 1,500 instructions a thread and sub-tile at 8 warps, whose latency
+// two warps a scheduler do not cover (0.8 instructions a clock)
+constexpr int OZ_WORKERS = 512;
 constexpr int OZ_THREADS = OZ_WORKERS + 32;  // plus one warp that issues the MMAs
-constexpr int OZ_SINK = 8;                   // columns a thread reads out at a time
+constexpr int OZ_SINK = 4;                   // columns a thread reads out at a time
 
 // One CTA: the 64 rows of C against up to OZ_CHUNK sub-tiles of 32 columns
 // of R.  C's slices stay in shared memory; R's are staged per sub-tile into
@@ -322,49 +325,48 @@ __device__ int oz_rows(OzSmem &sm, int kc, int ncols, CLoad cload, RLoad rload, 
   }
   // ---- A = the embedded C: real row 2rr = [Cr, -Ci], 2rr + 1 = [Ci, Cr]
   if (t < OZ_WORKERS) {
-    const int rr = t & 63, quarter = t >> 6;   // pivots [8 quarter, 8 quarter + 8) of row rr
-    double2 v[8];
+    const int rr = t & 63, part = t >> 6;   // pivots [4 part, 4 part + 4) of row rr
+    double2 v[4];
     int em = OZ_EMPTY;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int j = 8 * quarter + q;
+    for (int q = 0; q < 4; ++q) {
+      const int j = 4 * part + q;
       v[q] = j < kc ? cload(rr, j) : make_double2(0.0, 0.0);
       em = max(em, max(oz_exp(v[q].x), oz_exp(v[q].y)));
     }
     sm.red[t] = em;
     worker_sync();
-    const int er = max(max(sm.red[rr], sm.red[rr + 64]), max(sm.red[rr + 128], sm.red[rr + 192]));
-    if (quarter == 0) sm.eA[rr] = er;
+    int er = sm.red[rr];
+#pragma unroll
+    for (int o = 1; o < OZ_WORKERS / 64; ++o) er = max(er, sm.red[rr + 64 * o]);
+    if (part == 0) sm.eA[rr] = er;
     if (er > 1024) sm.bad = 1;
+    uint32_t re[4][OZ_S], im[4][OZ_S];
 #pragma unroll
-    for (int q0 = 0; q0 < 8; q0 += 4) {
-      uint32_t re[4][OZ_S], im[4][OZ_S];
+    for (int q = 0; q < 4; ++q) {
+      oz_slice(v[q].x, er, re[q]);
+      oz_slice(v[q].y, er, im[q]);
+    }
+    const int k0 = 8 * part;   // real K of this 16-byte chunk
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        oz_slice(v[q0 + q].x, er, re[q]);
-        oz_slice(v[q0 + q].y, er, im[q]);
-      }
-      const int k0 = 2 * (8 * quarter + q0);   // real K of this 16-byte chunk (a multiple of 8)
-#pragma unroll
-      for (int i = 0; i < OZ_S; ++i) {
-        uint4 w0, w1;
-        w0.x = re[0][i] | ((im[0][i] ^ 0x8000u) << 16);
-        w0.y = re[1][i] | ((im[1][i] ^ 0x8000u) << 16);
-        w0.z = re[2][i] | ((im[2][i] ^ 0x8000u) << 16);
-        w0.w = re[3][i] | ((im[3][i] ^ 0x8000u) << 16);
-        w1.x = im[0][i] | (re[0][i] << 16);
-        w1.y = im[1][i] | (re[1][i] << 16);
-        w1.z = im[2][i] | (re[2][i] << 16);
-        w1.w = im[3][i] | (re[3][i] << 16);
-        *reinterpret_cast<uint4 *>(sm.A[i] + op_off(2 * rr, k0)) = w0;
-        *reinterpret_cast<uint4 *>(sm.A[i] + op_off(2 * rr + 1, k0)) = w1;
-      }
+    for (int i = 0; i < OZ_S; ++i) {
+      uint4 w0, w1;
+      w0.x = re[0][i] | ((im[0][i] ^ 0x8000u) << 16);
+      w0.y = re[1][i] | ((im[1][i] ^ 0x8000u) << 16);
+      w0.z = re[2][i] | ((im[2][i] ^ 0x8000u) << 16);
+      w0.w = re[3][i] | ((im[3][i] ^ 0x8000u) << 16);
+      w1.x = im[0][i] | (re[0][i] << 16);
+      w1.y = im[1][i] | (re[1][i] << 16);
+      w1.z = im[2][i] | (re[2][i] << 16);
+      w1.w = im[3][i] | (re[3][i] << 16);
+      *reinterpret_cast<uint4 *>(sm.A[i] + op_off(2 * rr, k0)) = w0;
+      *reinterpret_cast<uint4 *>(sm.A[i] + op_off(2 * rr + 1, k0)) = w1;
     }
   }
   const int nsub = (ncols + OZ_NC - 1) / OZ_NC;
   const uint32_t idesc = tcx::instr_desc_f16(1, 128, OZ_NC);
   const int drow = (warp & 3) * 32 + lane, er = drow >> 1, comp = drow & 1;
-  const int hsel = warp >> 2;   // warps 0-3 read columns 0-15 of a sub-tile, warps 4-7 columns 16-31
+  const int hq = 8 * (warp >> 2);   // each four warps read 8 columns of a sub-tile, OZ_SINK at a time
   // read out sub-tile s: the 8 order sums of 16 columns at a time
   auto drain = [&](int s) {
     const int buf = s & 1;
@@ -375,31 +377,27 @@ __device__ int oz_rows(OzSmem &sm, int kc, int ncols, CLoad cload, RLoad rload, 
     if (!ok && lane == 0) atomicOr(&sm.bad, 2);
     if (!ok || (__shfl_sync(0xffffffffu, sm.bad, 0) & 1)) return;
 #pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      const int h = 16 * hsel + OZ_SINK * pass;
-      // the sink loads what it adds to first, then asks for the values
-      auto produce = [&](double (&add)[OZ_SINK]) {
+    for (int h = hq; h < hq + 8; h += OZ_SINK) {
+    // the sink loads what it adds to first, then asks for the values
+    auto produce = [&](double (&add)[OZ_SINK]) {
+      uint32_t vv[OZ_S][OZ_SINK];
+#pragma unroll
+      for (int g = 0; g < OZ_S; ++g)
+        tcx::tmem_ld4_async(sm.tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(256 * buf + OZ_NC * g + h), vv[g]);
+      tcx::tmem_wait(vv);
+#pragma unroll
+      for (int u = 0; u < OZ_SINK; ++u) {
         // pairs of orders first, in 32 bits: G_2q 2^7 + G_2q+1 stays below 2^31
-        int pr[4][OZ_SINK];
+        int pr[4];
 #pragma unroll
-        for (int g = 0; g < OZ_S; ++g) {
-          uint32_t vv[OZ_SINK];
-          tcx::tmem_ld8(sm.tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(256 * buf + OZ_NC * g + h), vv);
-#pragma unroll
-          for (int u = 0; u < OZ_SINK; ++u) {
-            const int G = __float2int_rn(__uint_as_float(vv[u]));
-            if (g & 1) pr[g >> 1][u] += G;
-            else pr[g >> 1][u] = G * 128;
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < OZ_SINK; ++u) {
-          const long long hi = (long long)pr[0][u] * (1ll << 14) + pr[1][u];
-          const long long lo = (long long)pr[2][u] * (1ll << 14) + pr[3][u];
-          add[u] = oz_value(hi * (1ll << 20) + (lo >> 8), sm.eA[er] + sm.eB[buf][h + u] - 55);
-        }
-      };
-      sink(er, OZ_NC * s + h, comp, produce);
+        for (int q = 0; q < 4; ++q)
+          pr[q] = __float2int_rn(__uint_as_float(vv[2 * q][u])) * 128 + __float2int_rn(__uint_as_float(vv[2 * q + 1][u]));
+        const long long hi = (long long)pr[0] * (1ll << 14) + pr[1];
+        const long long lo = (long long)pr[2] * (1ll << 14) + pr[3];
+        add[u] = oz_value(hi * (1ll << 20) + (lo >> 8), sm.eA[er] + sm.eB[buf][h + u] - 55);
+      }
+    };
+    sink(er, OZ_NC * s + h, comp, produce);
     }
   };
   tcx::fence_proxy_async();
@@ -439,13 +437,13 @@ __device__ int oz_rows(OzSmem &sm, int kc, int ncols, CLoad cload, RLoad rload, 
     }
     __syncwarp();
   } else {
-    const int cc = t & 31, oct = t >> 5;   // B staging: pivots [4 oct, 4 oct + 4) of column cc
-    double2 vn[4];                          // the next sub-tile's values, loaded ahead
+    const int cc = t & 31, part = t >> 5;   // B staging: pivots 2 part, 2 part + 1 of column cc
+    double2 vn[2];                          // the next sub-tile's values, loaded ahead
     auto load_b = [&](int s) {
       const int col = OZ_NC * s + cc;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int j = 4 * oct + q;
+      for (int q = 0; q < 2; ++q) {
+        const int j = 2 * part + q;
         vn[q] = (j < kc && col < ncols) ? rload(col, j) : make_double2(0.0, 0.0);
       }
     };
@@ -456,10 +454,10 @@ __device__ int oz_rows(OzSmem &sm, int kc, int ncols, CLoad cload, RLoad rload, 
       // ---- B(s): 32 columns as rows of K = [Rr, Ri] per pivot (its buffer
       // was last read by the MMAs of s - 2, finished before drain(s - 2))
       {
-        double2 v[4];
+        double2 v[2];
         int em = OZ_EMPTY;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < 2; ++q) {
           v[q] = vn[q];
           em = max(em, max(oz_exp(v[q].x), oz_exp(v[q].y)));
         }
@@ -468,25 +466,19 @@ __device__ int oz_rows(OzSmem &sm, int kc, int ncols, CLoad cload, RLoad rload, 
         worker_sync();
         int ec = sm.red[cc];
 #pragma unroll
-        for (int o = 1; o < 8; ++o) ec = max(ec, sm.red[cc + 32 * o]);
-        if (oct == 0) sm.eB[buf][cc] = ec;
+        for (int o = 1; o < OZ_WORKERS / 32; ++o) ec = max(ec, sm.red[cc + 32 * o]);
+        if (part == 0) sm.eB[buf][cc] = ec;
         if (ec > 1024) sm.bad = 1;
-        uint32_t re[4][OZ_S], im[4][OZ_S];
+        uint32_t re[2][OZ_S], im[2][OZ_S];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < 2; ++q) {
           oz_slice(v[q].x, ec, re[q]);
           oz_slice(v[q].y, ec, im[q]);
         }
-        const int k0 = 8 * oct;
 #pragma unroll
-        for (int i = 0; i < OZ_S; ++i) {
-          uint4 w;
-          w.x = re[0][i] | (im[0][i] << 16);
-          w.y = re[1][i] | (im[1][i] << 16);
-          w.z = re[2][i] | (im[2][i] << 16);
-          w.w = re[3][i] | (im[3][i] << 16);
-          *reinterpret_cast<uint4 *>(sm.B[buf][i] + op_off(cc, k0)) = w;
-        }
+        for (int i = 0; i < OZ_S; ++i)
+          *reinterpret_cast<uint2 *>(sm.B[buf][i] + op_off(cc, 4 * part)) =
+              make_uint2(re[0][i] | (im[0][i] << 16), re[1][i] | (im[1][i] << 16));
       }
       tcx::fence_proxy_async();
       tcx::mbar_arrive(smem_u32(&sm.bfull[buf]));
