@@ -292,12 +292,25 @@ void nn_conv(const float *in, int Cin, const float *w, const float *bias, float 
 // gw += weight gradient, gb += bias gradient (accumulated: zero them first)
 void nn_conv_wgrad(const float *in, int Cin, const float *gout, int Cout, int N, int H, int W, float *gw, float *gb,
                    cudaStream_t st);
-void nn_relu_mask(const float *y, float *g, int64_t n, cudaStream_t st);  // g = 0 where y <= 0
+// What a convolution does with each output besides bias and ReLU: out2 gets
+// the value, plus `add` where given (the sum with a skip connection, a
+// gradient kept before its mask); out gets it, zero where mask <= 0 (the
+// adjoint of the ReLU whose output mask is).
+struct ConvEpi {
+  const float *mask = nullptr, *add = nullptr;
+  float *out2 = nullptr;
+  __device__ __forceinline__ float apply(float r, int64_t i) const {
+    if (out2) out2[i] = add ? r + add[i] : r;
+    return mask && !(mask[i] > 0.f) ? 0.f : r;
+  }
+};
 void nn_pool2(const float *in, float *out, int64_t planes, int H, int W, cudaStream_t st);       // H, W of in
-void nn_pool2_bwd(const float *gout, float *gin, int64_t planes, int H, int W, cudaStream_t st);  // H, W of gin
+// g = (y > 0 ? g + pooling's adjoint of gout : 0), H, W of g
+void nn_pool2_bwd_add(const float *gout, const float *y, float *g, int64_t planes, int H, int W, cudaStream_t st);
 void nn_up2(const float *in, float *out, int64_t planes, int H, int W, cudaStream_t st);         // H, W of out
-void nn_up2_bwd(const float *gout, float *gin, int64_t planes, int H, int W, cudaStream_t st);   // H, W of gout
-void nn_axpy(const float *x, float *y, float a, int64_t n, cudaStream_t st);
+// gin = upsampling's adjoint of gout, zero where y <= 0; H, W of gout
+void nn_up2_bwd_mask(const float *gout, const float *y, float *gin, int64_t planes, int H, int W, cudaStream_t st);
+void nn_epilogue(float *out, const ConvEpi &e, int64_t n, cudaStream_t st);
 // loss += sum (p - t)^2 / n, g = 2 (p - t) / n
 void nn_mse(const float *p, const float *t, float *g, int64_t n, float *loss, cudaStream_t st);
 void nn_adam(float *w, float *wb, const float *g, float *m, float *v, int64_t n, float lr, int step, bool bf16,
@@ -334,8 +347,10 @@ int nn_num_sms();
 // gw += ..., gb += ... (accumulated with atomics: zero them first)
 void nn_conv_wgrad_tc(const float *in, int Cin, const float *gout, int Cout, int N, int H, int W, float *gw,
                       float *gb, int *flag, cudaStream_t st);
+// epi: see ConvEpi; up: the input is the H/2 x W/2 image, read through its
+// nearest 2x upsampling
 void nn_conv_tc(const float *in, int Cin, const uint16_t *wp, const float *bias, float *out, int Cout, int N, int H,
-                int W, bool relu, int *flag, cudaStream_t st, float *part);
+                int W, bool relu, int *flag, cudaStream_t st, float *part, const ConvEpi &epi, bool up);
 
 }  // namespace stdd
 

@@ -65,9 +65,12 @@ struct ConvTcArgs {
   int Cout, H, W, relu;
   int *flag;
   float *part;    // split-K: partial sums [gridDim.z][N][Cout][H][W], or null
+  ConvEpi epi;
+  int up;         // 1: the input is the upsampled image's source, H/2 x W/2 pixels
 };
 
-__global__ void __launch_bounds__(256) k_conv3x3_tc(ConvTcArgs a) {
+// EPI: with the epilogue's extra input and outputs, or an upsampled input
+template <bool EPI> __global__ void __launch_bounds__(256) k_conv3x3_tc(ConvTcArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
   const int wbytes = 288 * a.Npad;
   uint8_t *act0 = sm;
@@ -98,7 +101,9 @@ __global__ void __launch_bounds__(256) k_conv3x3_tc(ConvTcArgs a) {
   const uint32_t tmem = *tm;
   const uint32_t idesc = tcx::instr_desc_f16(1, 128, a.Npad);
   const int64_t plane = (int64_t)a.H * a.W;
-  const float *inb = a.in + (int64_t)n * a.Cin * plane;
+  const int up = EPI ? a.up : 0, Wi = a.W >> up;                  // the stored input's row
+  const int64_t iplane = (int64_t)(a.H >> up) * Wi;
+  const float *inb = a.in + (int64_t)n * a.Cin * iplane;
   bool ok = true;
   int issued = 0;   // chunks whose MMAs were committed
   // halo tile of 16 channels: items (plane cg, halo row, halo column), at
@@ -114,10 +119,9 @@ __global__ void __launch_bounds__(256) k_conv3x3_tc(ConvTcArgs a) {
       const int y = y0 - 1 + r / CT_HP, x = x0 - 1 + r % CT_HP;
       const bool ok_item = c < ce && it < 2 * CT_HP * CT_HP && y >= 0 && y < a.H && x >= 0 && x < a.W;
       const int ci0 = c * 16 + cg * 8;
+      const float *src = inb + (int64_t)ci0 * iplane + (int64_t)(y >> up) * Wi + (x >> up);
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        v[u][j] = (ok_item && ci0 + j < a.Cin) ? __ldg(inb + (int64_t)(ci0 + j) * plane + (int64_t)y * a.W + x)
-                                               : 0.f;
+      for (int j = 0; j < 8; ++j) v[u][j] = (ok_item && ci0 + j < a.Cin) ? __ldg(src + j * iplane) : 0.f;
     }
   };
   if (cb < ce) load_halo(cb);
@@ -197,9 +201,20 @@ __global__ void __launch_bounds__(256) k_conv3x3_tc(ConvTcArgs a) {
     const int y = y0 + (m >> 3), x = x0 + 8 * h + (m & 7);
     const bool store = y < a.H && x < a.W;
     const bool split = a.part != nullptr;
-    float *outp = (split ? a.part + (int64_t)blockIdx.z * gridDim.y * a.Cout * plane : a.out) +
-                  (int64_t)n * a.Cout * plane + (int64_t)y * a.W + x;
+    const int64_t at = (int64_t)n * a.Cout * plane + (int64_t)y * a.W + x;
+    float *outp = (split ? a.part + (int64_t)blockIdx.z * gridDim.y * a.Cout * plane : a.out) + at;
     for (int c0 = 0; c0 < a.Npad; c0 += 16) {
+      // what the epilogue reads is requested for all sixteen channels first
+      // (behind each other's stores they would wait one by one)
+      float mk[16], ad[16];
+      const bool mask = EPI && !split && a.epi.mask, add = EPI && !split && a.epi.add;
+      if (EPI)
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const bool in = store && c0 + u < a.Cout;
+        mk[u] = mask && in ? __ldg(a.epi.mask + at + (int64_t)(c0 + u) * plane) : 1.f;
+        ad[u] = add && in ? __ldg(a.epi.add + at + (int64_t)(c0 + u) * plane) : 0.f;
+      }
       uint32_t v[16];
       tcx::tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(h * a.Npad + c0), v);
 #pragma unroll
@@ -210,6 +225,8 @@ __global__ void __launch_bounds__(256) k_conv3x3_tc(ConvTcArgs a) {
           if (!split) {
             r += a.bias ? a.bias[co] : 0.f;
             if (a.relu) r = fmaxf(r, 0.f);
+            if (EPI && a.epi.out2) a.epi.out2[at + (int64_t)co * plane] = add ? r + ad[u] : r;
+            if (EPI && !(mk[u] > 0.f)) r = 0.f;
           }
           outp[(int64_t)co * plane] = r;
         }
@@ -225,12 +242,12 @@ __global__ void __launch_bounds__(256) k_conv3x3_tc(ConvTcArgs a) {
 
 // split-K epilogue: out = act(bias + sum over the slices, in slice order)
 __global__ void k_splitk_finish(const float *__restrict__ part, int ks, int64_t count, int64_t plane, int Cout,
-                                const float *__restrict__ bias, int relu, float *__restrict__ out) {
+                                const float *__restrict__ bias, int relu, float *__restrict__ out, ConvEpi epi) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
     float r = 0.f;
     for (int z = 0; z < ks; ++z) r += part[(int64_t)z * count + i];
     if (bias) r += bias[(int)((i / plane) % Cout)];
-    out[i] = relu ? fmaxf(r, 0.f) : r;
+    out[i] = epi.apply(relu ? fmaxf(r, 0.f) : r, i);
   }
 }
 
@@ -606,8 +623,11 @@ int nn_tc_nchunks(int Cin) { return (Cin + 15) / 16; }
 int64_t nn_tc_packed_elems(int Cin, int Cout) { return (int64_t)nn_tc_nchunks(Cin) * 9 * 2 * nn_tc_npad(Cout) * 8; }
 
 cudaError_t nn_tc_setup() {
-  const cudaError_t e =
-      cudaFuncSetAttribute(k_conv3x3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * CT_ACT + 576 * 256 + 64);
+  cudaError_t e = cudaFuncSetAttribute(k_conv3x3_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       2 * CT_ACT + 576 * 256 + 64);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(k_conv3x3_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           2 * CT_ACT + 576 * 256 + 64);
   if (e != cudaSuccess) return e;
   const cudaError_t e2 =
       cudaFuncSetAttribute(k_conv3x3_wgrad_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, WgCfg<32>::SMEM);
@@ -663,7 +683,7 @@ int nn_tc_ksplit(int Cin, int Cout, int N, int H, int W) {
 }
 
 void nn_conv_tc(const float *in, int Cin, const uint16_t *wp, const float *bias, float *out, int Cout, int N, int H,
-                int W, bool relu, int *flag, cudaStream_t st, float *part) {
+                int W, bool relu, int *flag, cudaStream_t st, float *part, const ConvEpi &epi, bool up) {
   ConvTcArgs a;
   a.in = in;
   a.Cin = Cin;
@@ -678,16 +698,19 @@ void nn_conv_tc(const float *in, int Cin, const uint16_t *wp, const float *bias,
   a.relu = relu ? 1 : 0;
   a.flag = flag;
   a.part = nullptr;
+  a.epi = epi;
+  a.up = up ? 1 : 0;
   const int tiles = ((W + CT_T - 1) / CT_T) * ((H + CT_T - 1) / CT_T);
   const size_t smem = 2 * CT_ACT + 2 * 288 * (size_t)a.Npad + 64;
   const int ks = part ? nn_tc_ksplit(Cin, Cout, N, H, W) : 1;
   a.part = ks > 1 ? part : nullptr;
-  k_conv3x3_tc<<<dim3(tiles, N, ks), 256, smem, st>>>(a);
+  if (up || epi.mask || epi.out2) k_conv3x3_tc<true><<<dim3(tiles, N, ks), 256, smem, st>>>(a);
+  else k_conv3x3_tc<false><<<dim3(tiles, N, ks), 256, smem, st>>>(a);
   count_launch();
   if (ks > 1) {
     const int64_t count = (int64_t)N * Cout * H * W;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((count + 255) / 256, 152 * 8));
-    k_splitk_finish<<<grid, 256, 0, st>>>(part, ks, count, (int64_t)H * W, Cout, bias, relu ? 1 : 0, out);
+    k_splitk_finish<<<grid, 256, 0, st>>>(part, ks, count, (int64_t)H * W, Cout, bias, relu ? 1 : 0, out, epi);
     count_launch();
   }
 }

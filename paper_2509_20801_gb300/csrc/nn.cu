@@ -200,15 +200,20 @@ struct stdd_nn {
   size_t layer_index(const Layer &ly) const { return (size_t)(&ly - layers.data()); }
 
   // out = conv(in) with layer ly (forward) or its input gradient (flip)
+  // epi: what else becomes of the outputs; up: `in` is the image of half the
+  // size that the layer sees upsampled (`scratch` holds that where the
+  // convolution cannot read through it)
   void conv(const float *in, const Layer &ly, float *out, int N, int H, int W, bool relu, bool flip,
-            cudaStream_t st) {
+            cudaStream_t st, const stdd::ConvEpi &epi = stdd::ConvEpi(), float *up_scratch = nullptr) {
     const int cin = flip ? ly.cout : ly.cin, cout = flip ? ly.cin : ly.cout;
     if (mode == STDD_NN_TC) {
       const size_t i = layer_index(ly);
       stdd::nn_conv_tc(in, cin, packed + (flip ? pk_bwd[i] : pk_fwd[i]), flip ? nullptr : wb.p + ly.boff, out, cout,
-                       N, H, W, relu, d_flag, st, act["ksplit"].p);
+                       N, H, W, relu, d_flag, st, act["ksplit"].p, epi, up_scratch != nullptr);
     } else {
-      stdd::nn_conv(in, cin, wb.p + ly.woff, flip ? nullptr : wb.p + ly.boff, out, cout, N, H, W, relu, flip, st);
+      stdd::nn_conv(up_scratch ? up_scratch : in, cin, wb.p + ly.woff, flip ? nullptr : wb.p + ly.boff, out, cout, N,
+                    H, W, relu, flip, st);
+      stdd::nn_epilogue(out, epi, (int64_t)N * cout * H * W, st);
     }
   }
 
@@ -287,18 +292,18 @@ struct stdd_nn {
   }
 
 
-  // forward pass; returns the output buffer (N x 2 x H x W)
-  void forward(int N, int H, int W, const float *in, float *out, cudaStream_t st) {
+  // forward pass into out (N x 2 x H x W); keep: a backward pass follows,
+  // which needs the upsampled images (the tensor-core convolutions read the
+  // small ones)
+  void forward(int N, int H, int W, const float *in, float *out, cudaStream_t st, bool keep = false) {
     check_shape(N, H, W);
     ensure_acts(N, H, W);
     for (int l = 0; l < L; ++l) {
       const int h = H >> l, wd = W >> l;
       const float *src = in;
-      int cin = 3;
       if (l > 0) {
         stdd::nn_pool2(A("skip", l - 1), A("pool", l), (int64_t)N * ch[l - 1], H >> (l - 1), W >> (l - 1), st);
         src = A("pool", l);
-        cin = ch[l - 1];
       }
       conv(src, encA(l), A("encA", l), N, h, wd, true, false, st);
       conv(A("encA", l), encB(l), A("skip", l), N, h, wd, true, false, st);
@@ -306,11 +311,11 @@ struct stdd_nn {
     for (int l = L - 2; l >= 0; --l) {
       const int h = H >> l, wd = W >> l;
       const float *deeper = (l + 1 == L - 1) ? A("skip", L - 1) : A("d", l + 1);
-      stdd::nn_up2(deeper, A("up", l), (int64_t)N * ch[l + 1], h, wd, st);
-      conv(A("up", l), decC(l), A("decC", l), N, h, wd, true, false, st);
-      const size_t cnt = sz(l, ch[l]);
-      NCK(cudaMemcpyAsync(A("sum", l), A("decC", l), cnt * sizeof(float), cudaMemcpyDeviceToDevice, st));
-      stdd::nn_axpy(A("skip", l), A("sum", l), 1.f, (int64_t)cnt, st);
+      if (keep || mode != STDD_NN_TC) stdd::nn_up2(deeper, A("up", l), (int64_t)N * ch[l + 1], h, wd, st);
+      stdd::ConvEpi skip;      // sum = decC + skip
+      skip.add = A("skip", l);
+      skip.out2 = A("sum", l);
+      conv(deeper, decC(l), A("decC", l), N, h, wd, true, false, st, skip, A("up", l));
       conv(A("sum", l), decD(l), A("d", l), N, h, wd, true, false, st);
     }
     const float *last = L > 1 ? A("d", 0) : A("skip", 0);
@@ -324,7 +329,7 @@ struct stdd_nn {
     check_shape(N, H, W);
     ensure_acts(N, H, W);  // sets the shapes sz() uses
     float *out = buf("out", sz(0, 2));
-    forward(N, H, W, in, out, st);
+    forward(N, H, W, in, out, st, true);
     NCK(cudaMemsetAsync(g.p, 0, nparams * sizeof(float), st));
     NCK(cudaMemsetAsync(loss.p, 0, sizeof(float), st));
     float *gout = act["gout"].p;
@@ -333,43 +338,41 @@ struct stdd_nn {
     // output layer
     const float *last = L > 1 ? A("d", 0) : A("skip", 0);
     wgrad(last, ch[0], gout, 2, N, H, W, g.p + outL().woff, g.p + outL().boff, st);
-    conv(gout, outL(), gd, N, H, W, false, true, st);  // grad of d_0
-    for (int l = 0; l < L; ++l)
-      NCK(cudaMemsetAsync(A("gskip", l), 0, sz(l, ch[l]) * sizeof(float), st));
-    if (L == 1) {
-      NCK(cudaMemcpyAsync(A("gskip", 0), gd, sz(0, ch[0]) * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    }
+    // a gradient is masked by its layer's ReLU where it is made
+    auto masked = [&](const float *y) {
+      stdd::ConvEpi e;
+      e.mask = y;
+      return e;
+    };
+    // grad of d_0 (of skip_0 in a network of one level)
+    conv(gout, outL(), L > 1 ? gd : A("gskip", 0), N, H, W, false, true, st, masked(last));
     // decoder, fine to coarse; gd holds the gradient w.r.t. d_l
     for (int l = 0; l <= L - 2; ++l) {
       const int h = H >> l, wd = W >> l;
-      const size_t cnt = sz(l, ch[l]);
-      stdd::nn_relu_mask(A("d", l), gd, (int64_t)cnt, st);
       wgrad(A("sum", l), ch[l], gd, ch[l], N, h, wd, g.p + decD(l).woff, g.p + decD(l).boff, st);
-      conv(gd, decD(l), t1, N, h, wd, false, true, st);  // grad of sum
-      stdd::nn_axpy(t1, A("gskip", l), 1.f, (int64_t)cnt, st);
-      stdd::nn_relu_mask(A("decC", l), t1, (int64_t)cnt, st);
+      // grad of sum: as it is the skip connection's share, masked decC's
+      stdd::ConvEpi both = masked(A("decC", l));
+      both.out2 = A("gskip", l);
+      conv(gd, decD(l), t1, N, h, wd, false, true, st, both);
       wgrad(A("up", l), ch[l + 1], t1, ch[l], N, h, wd, g.p + decC(l).woff, g.p + decC(l).boff, st);
       conv(t1, decC(l), t2, N, h, wd, false, true, st);  // grad of up
-      stdd::nn_up2_bwd(t2, gd, (int64_t)N * ch[l + 1], h, wd, st);  // grad of d_{l+1}
-      if (l + 1 == L - 1)
-        stdd::nn_axpy(gd, A("gskip", L - 1), 1.f, (int64_t)sz(L - 1, ch[L - 1]), st);
+      const bool deepest = l + 1 == L - 1;               // grad of d_{l+1} or of the deepest skip
+      stdd::nn_up2_bwd_mask(t2, A(deepest ? "skip" : "d", l + 1), deepest ? A("gskip", l + 1) : gd,
+                            (int64_t)N * ch[l + 1], h, wd, st);
     }
-    // encoder, coarse to fine
+    // encoder, coarse to fine; gskip_l holds the masked gradient w.r.t. skip_l
     for (int l = L - 1; l >= 0; --l) {
       const int h = H >> l, wd = W >> l;
-      const size_t cnt = sz(l, ch[l]);
       float *gs = A("gskip", l);
-      stdd::nn_relu_mask(A("skip", l), gs, (int64_t)cnt, st);
       wgrad(A("encA", l), ch[l], gs, ch[l], N, h, wd, g.p + encB(l).woff, g.p + encB(l).boff, st);
-      conv(gs, encB(l), t1, N, h, wd, false, true, st);  // grad of encA
-      stdd::nn_relu_mask(A("encA", l), t1, (int64_t)cnt, st);
+      conv(gs, encB(l), t1, N, h, wd, false, true, st, masked(A("encA", l)));  // grad of encA
       const float *src = l > 0 ? A("pool", l) : in;
       const int cin = l > 0 ? ch[l - 1] : 3;
       wgrad(src, cin, t1, ch[l], N, h, wd, g.p + encA(l).woff, g.p + encA(l).boff, st);
       if (l > 0) {
         conv(t1, encA(l), t2, N, h, wd, false, true, st);  // grad of pool
-        stdd::nn_pool2_bwd(t2, t1, (int64_t)N * cin, H >> (l - 1), W >> (l - 1), st);
-        stdd::nn_axpy(t1, A("gskip", l - 1), 1.f, (int64_t)sz(l - 1, ch[l - 1]), st);
+        stdd::nn_pool2_bwd_add(t2, A("skip", l - 1), A("gskip", l - 1), (int64_t)N * cin, H >> (l - 1),
+                               W >> (l - 1), st);
       }
     }
     NCK(cudaGetLastError());
