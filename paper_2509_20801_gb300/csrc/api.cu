@@ -1406,13 +1406,24 @@ void stdd_ctx::enqueue_minv_multiplicative(const std::vector<const double2 *> &v
     }
     return;
   }
+  std::vector<stdd::FieldBatch> batches;
+  for (int i = 0; i < na; ++i) {
+    if (i % stdd::FIELD_BATCH == 0) batches.push_back(stdd::FieldBatch{});
+    stdd::FieldBatch &B = batches.back();
+    B.v[B.n] = vs[i];
+    B.z[B.n++] = zs[i];
+  }
   for (const auto &gr : groups) {
-    for (int j = gr.first; j < gr.second; ++j)
-      for (int i = 0; i < na; ++i)
-        stdd::launch_restrict_residual_strip<R>(g, strips_host[perm[j]], vs[i], zs[i], slot(i), stream);
+    // strips of a group: one, or every second one from the first (perm)
+    const int first = perm[gr.first], count = gr.second - gr.first, step = count > 1 ? 2 : 1;
+    for (size_t k = 0; k < batches.size(); ++k)
+      stdd::launch_restrict_residual<R>(g, d_strips.as<StripDev>(), first, step, count, nloc_max, batches[k],
+                                        slot((int)k * stdd::FIELD_BATCH), nloc, stream);
     solve_range_levels<R>(gr.first, gr.second, na);
     for (int j = gr.first; j < gr.second; ++j)
-      for (int i = 0; i < na; ++i) stdd::launch_add_strip<R>(strips_host[perm[j]], ny, slot(i), zs[i], stream);
+      for (size_t k = 0; k < batches.size(); ++k)
+        stdd::launch_add_strip<R>(strips_host[perm[j]], ny, slot((int)k * stdd::FIELD_BATCH), nloc, batches[k],
+                                  stream);
   }
   CK(cudaGetLastError());
 }

@@ -217,12 +217,22 @@ void launch_synthesize_box(const StripDev *boxes_dev, int px, int py, int nx, in
 template <typename R>
 void launch_strip_norms(const StripDev *strips_dev, int nsub, int ny, const void *tloc, double *out,
                         cudaStream_t st);
-// one strip (multiplicative order): its local source R_s^I (v - A z), and
-// z += E_s e_s (tloc is the base of all strips' local fields)
+// (v, z) of the right-hand sides one launch works on
+constexpr int FIELD_BATCH = 16;
+struct FieldBatch {
+  int n;
+  const double2 *v[FIELD_BATCH];
+  double2 *z[FIELD_BATCH];
+};
+// multiplicative orders: the local sources R_s^I (v - A z) of the strips
+// first, first + step, ... (count of them; ids into strips_dev, none larger
+// than nloc_max nodes) into tloc, right-hand sides ldt elements apart; and
+// z += E_s e_s for one strip
 template <typename R>
-void launch_restrict_residual_strip(const GridDev &g, const StripDev &s, const double2 *v, const double2 *z,
-                                    void *tloc, cudaStream_t st);
-template <typename R> void launch_add_strip(const StripDev &s, int ny, const void *tloc, double2 *z, cudaStream_t st);
+void launch_restrict_residual(const GridDev &g, const StripDev *strips_dev, int first, int step, int count,
+                              int64_t nloc_max, const FieldBatch &B, void *tloc, int64_t ldt, cudaStream_t st);
+template <typename R>
+void launch_add_strip(const StripDev &s, int ny, const void *tloc, int64_t ldt, const FieldBatch &B, cudaStream_t st);
 // local strip k only: tloc_k = t (converted), and back
 template <typename R> void launch_to_local(const double2 *t, void *tloc, int64_t n, cudaStream_t st);
 template <typename R> void launch_from_local(const void *tloc, double2 *z, int64_t n, cudaStream_t st);

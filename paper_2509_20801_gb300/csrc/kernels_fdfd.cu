@@ -24,14 +24,9 @@ inline int grid_for(int64_t n) {
   return (int)std::min<int64_t>((n + TPB - 1) / TPB, 152 * 16);
 }
 
-__device__ __forceinline__ double2 apply_row_ij(const GridDev &g, const double2 *__restrict__ x, int64_t idx, int i,
-                                                int j) {
-  return grid_row(g, x, idx, i, j);
-}
-
 __device__ __forceinline__ double2 apply_row(const GridDev &g, const double2 *__restrict__ x, int64_t idx) {
   const int i = (int)(idx / g.ny), j = (int)(idx - (int64_t)i * g.ny);
-  return apply_row_ij(g, x, idx, i, j);
+  return grid_row(g, x, idx, i, j);
 }
 
 // y = A x, or y = b - A x (RES), column by column: a thread keeps its row j
@@ -57,12 +52,19 @@ __global__ void __launch_bounds__(COLT) k_stencil_cols(GridDev g, const double2 
     const bool has_s = j > 0, has_n = j < g.ny - 1;
     int64_t idx = (int64_t)i0 * g.ny + j;
     double2 w = i0 > 0 ? x[idx - g.ny] : zero, c = x[idx];
+    double2 bn = RES ? b[idx] : zero;
+    double kn = g.eps[idx];
     for (int i = i0; i < i1; ++i, idx += g.ny) {
       const double2 e = i < g.nx - 1 ? x[idx + g.ny] : zero;
       const double2 s = has_s ? x[idx - 1] : zero, n = has_n ? x[idx + 1] : zero;
       const double2 xm = g.cxm[i], xp = g.cxp[i];
-      const double2 bv = RES ? b[idx] : zero;
-      const double ke = g.eps[idx];
+      // b and the permittivity come from HBM: requested a column ahead
+      const double2 bv = bn;
+      const double ke = kn;
+      if (i + 1 < i1) {
+        if (RES) bn = b[idx + g.ny];
+        kn = g.eps[idx + g.ny];
+      }
       double2 acc;
       if (yreal && xm.y == 0.0 && xp.y == 0.0) {
         const double sg = RES ? -1.0 : 1.0;
@@ -206,27 +208,34 @@ __global__ void __launch_bounds__(TPB) k_synthesize_box(const StripDev *__restri
   }
 }
 
-// one strip s: t = R_s^I (v - A z) on its local box (zero off the owned
-// columns), the source of its local solve in the multiplicative order
+// the strips of a group (first, first + step, ...): t = R_s^I (v - A z) on
+// each local box (zero off the owned columns), the sources of their local
+// solves in the multiplicative orders; grid = (nodes, strips, right-hand
+// sides).  One launch for all (24 launches of 9.4 us each for three strips
+// and eight right-hand sides before).
 template <typename R>
-__global__ void __launch_bounds__(TPB) k_restrict_residual_strip(GridDev g, StripDev s, const double2 *__restrict__ v,
-                                                                 const double2 *__restrict__ z, void *tloc) {
+__global__ void __launch_bounds__(TPB) k_restrict_residual(GridDev g, const StripDev *__restrict__ strips, int first,
+                                                           int step, FieldBatch B, void *tloc, int64_t ldt) {
   using C = typename CT<R>::T;
-  const int64_t nl = (int64_t)(s.x1 - s.x0) * g.ny;
-  const int64_t lo = (int64_t)(s.c0 - s.x0) * g.ny, hi = (int64_t)(s.c1 - s.x0) * g.ny;
-  const int64_t g0 = (int64_t)s.x0 * g.ny;
-  C *t = reinterpret_cast<C *>(tloc) + s.vec_off;
-  for (int64_t l = (int64_t)blockIdx.x * TPB + threadIdx.x; l < nl; l += (int64_t)gridDim.x * TPB)
-    t[l] = (l >= lo && l < hi) ? to_c(csub(v[g0 + l], apply_row(g, z, g0 + l)), C()) : czero<C>();
+  const StripDev s = strips[first + step * blockIdx.y];
+  const double2 *__restrict__ v = B.v[blockIdx.z], *__restrict__ z = B.z[blockIdx.z];
+  const int nl = (s.x1 - s.x0) * g.ny;
+  C *t = reinterpret_cast<C *>(tloc) + blockIdx.z * ldt + s.vec_off;
+  for (int l = blockIdx.x * TPB + threadIdx.x; l < nl; l += gridDim.x * TPB) {
+    const int lx = l / g.ny, i = s.x0 + lx, j = l - lx * g.ny;
+    const int64_t at = (int64_t)s.x0 * g.ny + l;
+    t[l] = i >= s.c0 && i < s.c1 ? to_c(csub(v[at], grid_row(g, z, at, i, j)), C()) : czero<C>();
+  }
 }
 
-// z += E_s e_s: the strip's full local field added on its local box
+// z += E_s e_s: one strip's full local fields added on its local box, every
+// right-hand side (boxes of a colour may overlap: strips one after another)
 template <typename R>
-__global__ void __launch_bounds__(TPB) k_add_strip(StripDev s, int ny, const void *tloc, double2 *__restrict__ z) {
+__global__ void __launch_bounds__(TPB) k_add_strip(StripDev s, int ny, const void *tloc, int64_t ldt, FieldBatch B) {
   using C = typename CT<R>::T;
-  const C *t = reinterpret_cast<const C *>(tloc) + s.vec_off;
+  const C *t = reinterpret_cast<const C *>(tloc) + blockIdx.y * ldt + s.vec_off;
   const int64_t nl = (int64_t)(s.x1 - s.x0) * ny;
-  double2 *zs = z + (int64_t)s.x0 * ny;
+  double2 *zs = B.z[blockIdx.y] + (int64_t)s.x0 * ny;
   for (int64_t l = (int64_t)blockIdx.x * TPB + threadIdx.x; l < nl; l += (int64_t)gridDim.x * TPB)
     zs[l] = cadd(zs[l], to_d(t[l]));
 }
@@ -457,21 +466,23 @@ template <typename R> void launch_from_local(const void *tloc, double2 *z, int64
 }
 
 template <typename R>
-void launch_restrict_residual_strip(const GridDev &g, const StripDev &s, const double2 *v, const double2 *z,
-                                    void *tloc, cudaStream_t st) {
-  k_restrict_residual_strip<R><<<grid_for((int64_t)(s.x1 - s.x0) * g.ny), TPB, 0, st>>>(g, s, v, z, tloc);
+void launch_restrict_residual(const GridDev &g, const StripDev *strips_dev, int first, int step, int count,
+                              int64_t nloc_max, const FieldBatch &B, void *tloc, int64_t ldt, cudaStream_t st) {
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((nloc_max + TPB - 1) / TPB, 152 * 8));
+  k_restrict_residual<R><<<dim3(blocks, count, B.n), TPB, 0, st>>>(g, strips_dev, first, step, B, tloc, ldt);
   count_launch();
 }
-template <typename R> void launch_add_strip(const StripDev &s, int ny, const void *tloc, double2 *z, cudaStream_t st) {
-  k_add_strip<R><<<grid_for((int64_t)(s.x1 - s.x0) * ny), TPB, 0, st>>>(s, ny, tloc, z);
+template <typename R>
+void launch_add_strip(const StripDev &s, int ny, const void *tloc, int64_t ldt, const FieldBatch &B, cudaStream_t st) {
+  k_add_strip<R><<<dim3(grid_for((int64_t)(s.x1 - s.x0) * ny), B.n), TPB, 0, st>>>(s, ny, tloc, ldt, B);
   count_launch();
 }
-template void launch_restrict_residual_strip<double>(const GridDev &, const StripDev &, const double2 *,
-                                                     const double2 *, void *, cudaStream_t);
-template void launch_restrict_residual_strip<float>(const GridDev &, const StripDev &, const double2 *,
-                                                    const double2 *, void *, cudaStream_t);
-template void launch_add_strip<double>(const StripDev &, int, const void *, double2 *, cudaStream_t);
-template void launch_add_strip<float>(const StripDev &, int, const void *, double2 *, cudaStream_t);
+template void launch_restrict_residual<double>(const GridDev &, const StripDev *, int, int, int, int64_t,
+                                               const FieldBatch &, void *, int64_t, cudaStream_t);
+template void launch_restrict_residual<float>(const GridDev &, const StripDev *, int, int, int, int64_t,
+                                              const FieldBatch &, void *, int64_t, cudaStream_t);
+template void launch_add_strip<double>(const StripDev &, int, const void *, int64_t, const FieldBatch &, cudaStream_t);
+template void launch_add_strip<float>(const StripDev &, int, const void *, int64_t, const FieldBatch &, cudaStream_t);
 
 template <typename R>
 void launch_restrict_band(const StripDev *strips_dev, int nsub, int64_t nloc_max, int ny, const int64_t *colband,
