@@ -1080,7 +1080,7 @@ __device__ __forceinline__ void row_chains(const C *__restrict__ M, int64_t ld, 
 // of two its column was scaled by; sink(chain, sums) receives each chain's
 // sums, sums[q][t] the lane's component (lane % 2) of its row (fx_row) of tile t.
 template <int MT, int NR, typename Gather, typename Expo, typename Sink>
-__device__ __forceinline__ void fx_chains(FxRows<MT> &f, int r0, int k0, int k1, int lane, const FxLane &fl,
+__device__ __forceinline__ void fx_chains(FxRows<MT, NR> &f, int r0, int k0, int k1, int lane, const FxLane &fl,
                                           ulonglong2 (*xs)[FX_COLS], Gather gather, Expo expo, Sink sink) {
   const int cend = f.cend;
   double2 vn[NR];
@@ -1116,8 +1116,6 @@ __device__ __forceinline__ void fx_chains(FxRows<MT> &f, int r0, int k0, int k1,
 }
 // row of a 16-row tile whose sum a lane of fx_chain holds
 __device__ __forceinline__ int fx_row(int lane) { return 8 * ((lane >> 1) & 1) + (lane >> 2); }
-// component lane % 2 of v
-__device__ __forceinline__ double fx_part(double2 v, int lane) { return (lane & 1) ? v.y : v.x; }
 
 // Factor blocks of a level's eliminated large fronts to fixed point, in place: one
 // warp per 32 rows of a chain, lane = row, 32 columns in registers.  Reads
@@ -1239,6 +1237,20 @@ __device__ __forceinline__ C wsrc_children(const WSrc<C> &s, int k, int q, C w) 
       if (t >= 0) w = cadd(w, s.uc[ci][(int64_t)q * s.bc[ci] + t]);
     }
   return w;
+}
+// the children's update vectors at position k, component comp alone: one
+// addition where both children have the position, none otherwise
+__device__ __forceinline__ double wsrc_children_part(const WSrc<double2> &s, int k, int q, int comp) {
+  double v[2] = {0.0, 0.0};
+  bool has[2] = {false, false};
+#pragma unroll
+  for (int ci = 0; ci < 2; ++ci)
+    if (s.uc[ci]) {
+      const int t = s.inv[ci][k];
+      has[ci] = t >= 0;
+      if (has[ci]) v[ci] = reinterpret_cast<const double *>(s.uc[ci] + (int64_t)q * s.bc[ci] + t)[comp];
+    }
+  return has[0] && has[1] ? v[0] + v[1] : has[1] ? v[1] : v[0];
 }
 // pivot position k < p; *gi = its slot in tloc / wloc
 template <typename C>
@@ -1470,43 +1482,36 @@ template <int MT, int NR> struct FxFold {
   __device__ __forceinline__ void add(int q, int t, int k, int nk, double s) {
     constexpr int PER = MF_SEG / FX_COLS;
     seg[q][t] = k % PER == 0 ? s : seg[q][t] + s;
-    if (k % PER == PER - 1 || k == nk - 1) total[q][t] += seg[q][t];
+    if (k % PER == PER - 1 || k == nk - 1) total[q][t] = k < PER ? seg[q][t] : total[q][t] + seg[q][t];
   }
 };
+
+// A warp's copy of its front's record in shared memory: read once, in one
+// coalesced request, and from there where a field is needed -- the fused
+// upward products otherwise hold some thirty registers of it.
+__device__ __forceinline__ void warp_record(const MfArgs &a, int front, SweepFront *rec, int lane) {
+  static_assert(sizeof(SweepFront) == 128, "eight lanes of sixteen bytes");
+  __syncwarp();
+  if (lane < 8) reinterpret_cast<uint4 *>(rec)[lane] = reinterpret_cast<const uint4 *>(a.sweep + front)[lane];
+  __syncwarp();
+}
 
 template <int MT, int NR, bool FUSED, bool PDL>
 __device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                             int nrhs, int64_t ldt, int vb, double *part,
-                                            ulonglong2 (*xs)[FX_COLS]) {
+                                            ulonglong2 (*xs)[FX_COLS], SweepFront *rec) {
   const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ipc = 8 / split, il = g / split, sidx = g - il * split;
   const int it = vb * ipc + il;
   const bool active = it < nitems;
   const FxLane fl(lane);
   int p = 0, b = 0, r0 = 0, k0 = 0, k1 = 0, nk = 0;
-  const double2 *G = nullptr;
-  const short *E = nullptr;
-  const int *nodes = nullptr, *pc = nullptr;
-  int64_t voff = 0;
-  double2 *u = nullptr;
-  WSrc<double2> src;
-  bool writer = false;
   if (active) {
     const int2 item = items[it];
-    const SweepFront f = a.sweep[item.x];
-    p = f.p;
-    b = f.b;
-    voff = f.voff;
-    if (FUSED) {
-      src = wsrc_make(a, f, nrhs);
-      writer = item.y == 0;
-    }
-    G = reinterpret_cast<const double2 *>(a.fac) + f.up;   // -G21, b x p, ld b
-    E = a.fexp + f.eup;
+    warp_record(a, item.x, rec, lane);
+    p = rec->p;
+    b = rec->b;
     r0 = item.y * 16 * MT;
-    nodes = a.nodes + f.nodes;
-    u = reinterpret_cast<double2 *>(a.ub_cur) + f.u * nrhs;
-    if (a.pcol) pc = a.pcol + f.piv;
     nk = (p + FX_COLS - 1) / FX_COLS;
     k0 = sidx * nk / split;
     k1 = (sidx + 1) * nk / split;
@@ -1514,8 +1519,10 @@ __device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restr
   double2 *wl = reinterpret_cast<double2 *>(a.wloc);
   double *mine = part + (int64_t)il * mf_max_chains(16, 16 * MT, split, NR) * NR * MT * 32 + lane;
   for (int q0 = blockIdx.y * NR; q0 < nrhs; q0 += gridDim.y * NR) {
-    FxRows<MT> f;
-    f.start(G, E, r0, b, k0 * FX_COLS, min(p, k1 * FX_COLS), lane);
+    FxRows<MT, NR> f;
+    if (active)   // -G21, b x p, ld b
+      f.start(reinterpret_cast<const double2 *>(a.fac) + rec->up, a.fexp + rec->eup, r0, b, k0 * FX_COLS,
+              min(p, k1 * FX_COLS), lane);
     if (PDL) level_wait();
     double w0[NR][MT];     // the children's update vectors at the item's rows
 #pragma unroll
@@ -1526,17 +1533,19 @@ __device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restr
         const int64_t at = (int64_t)(q0 + q) * b + r;
         w0[q][t] = 0.0;
         if (sidx == 0 && r < b && q0 + q < nrhs)
-          w0[q][t] = fx_part(FUSED ? wsrc_children(src, p + r, q0 + q, czero<double2>()) : u[at], lane);
+          w0[q][t] = FUSED ? wsrc_children_part(wsrc_make(a, *rec, nrhs), p + r, q0 + q, lane & 1)
+                           : reinterpret_cast<const double *>(a.ub_cur)[2 * (rec->u * nrhs + at) + (lane & 1)];
       }
     FxFold<MT, NR> fold;
     fold.clear();
     if (k0 < k1) {
       auto gather = [&](int j, int q) {
         if (q0 + q >= nrhs) return czero<double2>();
-        if (!FUSED) return wl[(q0 + q) * ldt + voff + nodes[pc ? pc[j] : j]];
+        const int k = a.pcol ? a.pcol[rec->piv + j] : j;
+        if (!FUSED) return wl[(q0 + q) * ldt + rec->voff + a.nodes[rec->nodes + k]];
         int64_t gi;
-        const double2 w = wsrc_pivot(a, src, pc ? pc[j] : j, q0 + q, ldt, &gi);
-        if (writer) wl[gi] = w;
+        const double2 w = wsrc_pivot(a, wsrc_make(a, *rec, nrhs), k, q0 + q, ldt, &gi);
+        if (r0 == 0) wl[gi] = w;      // the front's first rows store w_p for the way down
         return w;
       };
       fx_chains<MT, NR>(f, r0, k0, k1, lane, fl, xs, gather, [](int) { return 0; },
@@ -1562,7 +1571,8 @@ __device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restr
 #pragma unroll
           for (int q = 0; q < NR; ++q)
             if (q0 + q < nrhs)
-              reinterpret_cast<double *>(u)[2 * ((int64_t)(q0 + q) * b + r) + (lane & 1)] = w0[q][t] + fold.total[q][t];
+              reinterpret_cast<double *>(a.ub_cur)[2 * (rec->u * nrhs + (int64_t)(q0 + q) * b + r) + (lane & 1)] =
+                  w0[q][t] + fold.total[q][t];
       }
     }
     if (split > 1) __syncthreads();
@@ -1572,28 +1582,19 @@ __device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restr
 template <int MT, int NR, bool PDL>
 __device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                               int nrhs, int64_t ldt, int vb, double *part,
-                                              ulonglong2 (*xs)[FX_COLS]) {
+                                              ulonglong2 (*xs)[FX_COLS], SweepFront *rec) {
   const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ipc = 8 / split, il = g / split, sidx = g - il * split;
   const int it = vb * ipc + il;
   const bool active = it < nitems;
   const FxLane fl(lane);
   int p = 0, n = 0, r0 = 0, k0 = 0, k1 = 0, nk = 0;
-  const double2 *Fm = nullptr;
-  const short *E = nullptr;
-  const int *nodes = nullptr, *pc = nullptr;
-  int64_t voff = 0;
   if (active) {
     const int2 item = items[it];
-    const SweepFront f = a.sweep[item.x];
-    p = f.p;
-    n = p + f.b;
-    voff = f.voff;
-    Fm = reinterpret_cast<const double2 *>(a.fac) + f.down;   // p x n, ld p
-    E = a.fexp + f.edown;
+    warp_record(a, item.x, rec, lane);
+    p = rec->p;
+    n = p + rec->b;
     r0 = item.y * 16 * MT;
-    nodes = a.nodes + f.nodes;
-    if (a.pcol) pc = a.pcol + f.piv;
     nk = (n + FX_COLS - 1) / FX_COLS;
     k0 = sidx * nk / split;
     k1 = (sidx + 1) * nk / split;
@@ -1602,16 +1603,19 @@ __device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__res
   const double2 *wl = reinterpret_cast<const double2 *>(a.wloc);
   double *mine = part + (int64_t)il * mf_max_chains(16, 16 * MT, split, NR) * NR * MT * 32 + lane;
   for (int q0 = blockIdx.y * NR; q0 < nrhs; q0 += gridDim.y * NR) {
-    FxRows<MT> f;
-    f.start(Fm, E, r0, p, k0 * FX_COLS, min(n, k1 * FX_COLS), lane);
+    FxRows<MT, NR> f;
+    if (active)   // p x n, ld p
+      f.start(reinterpret_cast<const double2 *>(a.fac) + rec->down, a.fexp + rec->edown, r0, p, k0 * FX_COLS,
+              min(n, k1 * FX_COLS), lane);
     if (PDL) level_wait();
     FxFold<MT, NR> fold;
     fold.clear();
     if (k0 < k1) {
       auto gather = [&](int c, int q) {
         if (q0 + q >= nrhs) return czero<double2>();
-        const int64_t base = (q0 + q) * ldt + voff;
-        return c < p ? wl[base + nodes[pc ? pc[c] : c]] : cneg(tv[base + nodes[c]]);
+        const int64_t base = (q0 + q) * ldt + rec->voff;
+        const int k = c < p && a.pcol ? a.pcol[rec->piv + c] : c, node = a.nodes[rec->nodes + k];
+        return c < p ? wl[base + node] : cneg(tv[base + node]);
       };
       fx_chains<MT, NR>(f, r0, k0, k1, lane, fl, xs, gather,
                         [&](int c) { return c < p ? a.fx_scale : 0; },
@@ -1637,7 +1641,8 @@ __device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__res
 #pragma unroll
           for (int q = 0; q < NR; ++q)
             if (q0 + q < nrhs)
-              reinterpret_cast<double *>(tv)[2 * ((q0 + q) * ldt + voff + nodes[r]) + (lane & 1)] = fold.total[q][t];
+              reinterpret_cast<double *>(
+                  tv)[2 * ((q0 + q) * ldt + rec->voff + a.nodes[rec->nodes + r]) + (lane & 1)] = fold.total[q][t];
       }
     }
     if (split > 1) __syncthreads();
@@ -1653,13 +1658,15 @@ template <typename R> __host__ __device__ constexpr int block_items(int rows) {
 // one (virtual) block of products of either precision; `part` holds the
 // segment sums of split items, the warps' vector words follow it
 template <typename R, int NR>
-constexpr int SWEEP_SMEM = MF_PART_BYTES / (2 * sizeof(R)) + (sizeof(R) == 8 ? 8 * NR * FX_COLS : 0);
+constexpr int SWEEP_SMEM = MF_PART_BYTES / (2 * sizeof(R)) + (sizeof(R) == 8 ? 8 * NR * FX_COLS + 8 * (int)sizeof(SweepFront) / 16 : 0);
 template <typename R, int ROWS, int NR, bool FUSED, bool PDL>
 __device__ __forceinline__ void up_any(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                        int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
   if constexpr (sizeof(R) == 8) {
     auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_PART_BYTES / sizeof(double2)) + (threadIdx.x >> 5) * NR;
-    up_block_fx<ROWS / 16, NR, FUSED, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs);
+    auto rec = reinterpret_cast<SweepFront *>(part + MF_PART_BYTES / sizeof(double2) + 8 * NR * FX_COLS) + (threadIdx.x >> 5);
+    up_block_fx<ROWS / 16, NR, FUSED, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs,
+                                        rec);
   } else {
     if (PDL) level_wait();
     up_block<R, ROWS, NR, FUSED>(a, items, nitems, split, nrhs, ldt, vb, part);
@@ -1670,7 +1677,9 @@ __device__ __forceinline__ void down_any(const MfArgs &a, const int2 *__restrict
                                          int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
   if constexpr (sizeof(R) == 8) {
     auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_PART_BYTES / sizeof(double2)) + (threadIdx.x >> 5) * NR;
-    down_block_fx<ROWS / 16, NR, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs);
+    auto rec = reinterpret_cast<SweepFront *>(part + MF_PART_BYTES / sizeof(double2) + 8 * NR * FX_COLS) + (threadIdx.x >> 5);
+    down_block_fx<ROWS / 16, NR, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs,
+                                        rec);
   } else {
     if (PDL) level_wait();
     down_block<R, ROWS, NR>(a, items, nitems, split, nrhs, ldt, vb, part);
@@ -1741,7 +1750,7 @@ __global__ void __launch_bounds__(256) mf_seg_partial(MfArgs a, const int2 *__re
     const FxLane fl(lane);
     const short *E = a.fexp + f.exp_off + (UP ? (int64_t)p * ((n + FX_COLS - 1) / FX_COLS) : 0);
     double *out = reinterpret_cast<double *>(a.segpart) + u * 64 + 2 * fx_row(lane) + (lane & 1);
-    FxRows<2> walk;
+    FxRows<2, 1> walk;
     walk.start(M, E, item.y * 32, ld, c0, c1, lane);
     level_wait();
     fx_chains<2, 1>(walk, item.y * 32, sg, sg + 1, lane, fl, xs[warp], gather,

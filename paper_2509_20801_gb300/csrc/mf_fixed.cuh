@@ -142,8 +142,9 @@ __host__ __device__ __forceinline__ int64_t fx_exps(int p, int b) {
 // column c at M[c rows + r0 + i]) with the rows' exponents E, chain by chain.
 // The matrix loads run AHEAD groups of four columns in front of the products,
 // across chains and before the chain's vector values have arrived.
-template <int MT> struct FxRows {
-  static constexpr int AHEAD = MT == 2 ? 2 : 4;
+template <int MT, int NR> struct FxRows {
+  // (two right-hand sides: their accumulators take the registers)
+  static constexpr int AHEAD = (MT == 2 ? 2 : 4) / NR;
   const uint4 *row[2 * MT];
   int64_t ld;
   const short *E;
@@ -193,7 +194,7 @@ __device__ __forceinline__ double fx_value(long long hi, long long lo, int e) {
 // zero past the end; ex[q]: their exponent.  out[q][t]: of row 16 t + lane /
 // 4 + 8 (lane / 2 % 2), component lane % 2.
 template <int MT, int NR>
-__device__ __forceinline__ void fx_chain(FxRows<MT> &f, int r0, int c0, int lane, const FxLane &fl,
+__device__ __forceinline__ void fx_chain(FxRows<MT, NR> &f, int r0, int c0, int lane, const FxLane &fl,
                                          const ulonglong2 (*xs)[FX_COLS], const int (&ex)[NR],
                                          double (&out)[NR][MT]) {
   const int g = lane >> 2, c = lane & 3;
