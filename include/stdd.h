@@ -367,8 +367,8 @@ stdd_status stdd_set_profiling(stdd_ctx *ctx, int level);
  *                     0: one launch per level; k = 1..8: the cooperative
  *                     grid holds k blocks per SM (at most what fits); -1: 2
  *                     for complex64 factors, 0 for complex128 ones (whose
- *                     products are FP64-bound per warp and run faster in the
- *                     per-level kernels' deeper load pipelines).  Same
+ *                     products run faster in the per-level kernels, which
+ *                     have more registers and overlapped launches).  Same
  *                     arithmetic, same results.
  *   STDD_OPT_SWEEP_WAIT (default 0 = 4,194,304): polls a block spends at one
  *                     grid barrier of a persistent sweep before it gives up;
@@ -431,8 +431,7 @@ stdd_status stdd_set_profiling(stdd_ctx *ctx, int level);
  *                     by the autotuner; 1, 2, 4, 8: that many warps of one
  *                     block per item; 16: one warp per (item, segment)
  *                     anywhere on the GPU, the segment sums added by a
- *                     second launch (32-row items; the FP64 pipe of one SM
- *                     no longer bounds a root-level item).  Every choice
+ *                     second launch (32-row items).  Every choice
  *                     gives the same sums in the same order: results do not
  *                     change.  Applied at the next stdd_factor. */
 enum {

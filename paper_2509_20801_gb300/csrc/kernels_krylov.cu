@@ -66,7 +66,8 @@ template <int N> __device__ __forceinline__ double warp_sums(double (&v)[N], int
 // over the warps is paid once for a chunk of some thousand elements; with all
 // groups in every block, chunks of two elements a thread and a block-wide sum
 // for each component, the reductions took two thirds of the time (262,144
-// nodes, 40 vectors: 212 us; the FP64 pipe needs 76).
+// nodes, 40 vectors: 212 us; the FP64 pipe needs 76).  Eight bases of 262,144
+// nodes and some 25 vectors now take 397 us in one launch, the pipe's time.
 __global__ void __launch_bounds__(TPB) k_mdot(KrylovBatch B, const double2 *__restrict__ Vb, int64_t ldv, int m,
                                               int64_t n, double2 *__restrict__ partial, int self_norm) {
   __shared__ double sh[TPB / 32][2 * GROUP + 1];
@@ -145,7 +146,8 @@ __global__ void k_reduce_r(KrylovBatch B, const double *__restrict__ partial, in
 
 // w -= sum_i h[z][i] V_i and the partial sums of ||w||^2; grid = (chunks,
 // bases).  Four vectors' values are in flight at a time (72 us for 40 vectors
-// of 262,144 nodes: the FP64 pipe's 76 % of the time it needs at its peak).
+// of 262,144 nodes; 320 us for eight bases of some 25 vectors in one launch):
+// four multiply-adds an entry at the FP64 pipe's rate.
 __global__ void __launch_bounds__(TPB) k_maxpy_norm(KrylovBatch B, double2 *__restrict__ Vb, int64_t ldv, int m,
                                                     const double2 *__restrict__ h, int64_t ldh, int64_t n,
                                                     double *__restrict__ partial) {

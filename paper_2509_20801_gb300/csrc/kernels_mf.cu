@@ -180,7 +180,10 @@ __device__ __forceinline__ C front_entry(const MfArgs &a, const FrontDev &f, con
   return out;
 }
 
-// Large fronts (n > MF_SMALL): write the assembled front to its storage.
+// Large fronts (n > MF_SMALL): write the assembled front to its storage.  A
+// thread keeps its row and walks columns: the column's coefficients and child
+// positions are the same for the whole warp (1024 x 512 in 4 strips: 1.21 ms
+// in all, 1.68 ms with a division and every look-up per entry).
 template <typename R>
 __global__ void __launch_bounds__(256) mf_assemble(MfArgs a, int f0) {
   using C = typename CT<R>::T;
@@ -298,8 +301,9 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
   // A box without children (symmetric form): each border node couples to one
   // pivot, F12(:, c) = a_c e_k(c), and F22 is zero, so only F11 is swept --
   // H12(:, c) = Finv(:, k(c)) a_c, S = - a_r Finv(k(r), k(c)) a_c -- a third
-  // of the sweep's multiply-adds at 16 pivots and 16 border nodes (32,768
-  // such fronts: 2.47 ms when the whole front was swept, FP64-pipe bound).
+  // of the sweep's multiply-adds at 16 pivots and 16 border nodes.  FP64-pipe
+  // bound: the fronts of up to 32 rows of a 1024 x 512 grid in 4 strips took
+  // 3.04 ms when every front was swept whole, 1.97 ms so.
   const bool leaf = sym && !has[0] && !has[1];
   const int m = leaf ? p : n;                       // rows and columns swept
   const int lds = leaf ? (p | 1) : ld;
@@ -607,10 +611,10 @@ __global__ void __launch_bounds__(MF_PANEL_THREADS) mf_gj_row_mirror(MfArgs a, i
 // warp of its own takes the next pivot through the update and forms its
 // reciprocal while the others still update.  (One triangle, mirrored in the
 // symmetric form, takes no less: its rows end within warps.)
-// 104 us a block of 32 in complex128 with 128 threads, the pivot row and
-// column on branches of their own -- the FP64 pipe pays a branch that one lane
-// takes like all -- and the correctly rounded reciprocal and its statistics
-// between two barriers.
+// 63 us a block of 32 in complex128; 104 us with 128 threads, the pivot row
+// and column on branches of their own -- the FP64 pipe pays a branch that one
+// lane takes like all -- and the correctly rounded reciprocal and its
+// statistics between two barriers.
 // The blocks past the first of a front (symmetric form) mirror the previous
 // step's pivot rows: the column panel of this step needs both, and mirroring
 // takes a fraction of the inverse's time (23 us as a launch of its own).
@@ -1001,9 +1005,11 @@ __global__ void __launch_bounds__(256) mf_gj_update(MfArgs a, int f0, int k) {
 // order, so the result does not depend on how many row groups share an item
 // (split) -- split only decides which group computes which segments.  With
 // split > 1 the segment sums meet in shared memory and the first group of
-// the item adds them.  Column values are gathered ROWS at a time (one per
-// lane) and broadcast by shuffles; each lane keeps MF_UNROLL matrix loads in
-// flight.
+// the item adds them.  complex64: column values are gathered ROWS at a time
+// (one per lane) and broadcast by shuffles, and each lane keeps a chunk's
+// matrix loads in flight.  complex128: digit products of whole chains on the
+// tensor cores (mf_fixed.cuh), a warp per (front, chunk of ROWS rows, run of
+// chains) at both chunk heights.
 template <int W, typename C> __device__ __forceinline__ C shfl_w(unsigned mask, C v, int src) {
   v.x = __shfl_sync(mask, v.x, src, W);
   v.y = __shfl_sync(mask, v.y, src, W);
@@ -1707,9 +1713,9 @@ __global__ void __launch_bounds__(256, 2) mf_down(MfArgs a, const int2 *__restri
 // chain) anywhere in the grid writes the chain's sum per row, and a second
 // launch folds the chains into segment sums and the segment sums into the
 // total, in column order -- the association seg_dot and the in-block
-// split use, so the choice between them changes no result.  At the top tree levels a few fronts
-// carry a whole phase; an in-block split keeps an item on one SM, whose FP64
-// pipe then sets the phase time.
+// split use, so the choice between them changes no result.  At the top tree
+// levels a few fronts carry a whole phase; an in-block split keeps an item on
+// one SM.
 template <typename R, bool UP, bool FUSED>
 __global__ void __launch_bounds__(256) mf_seg_partial(MfArgs a, const int2 *__restrict__ items, int nitems,
                                                       int nsubmax, int64_t ldt) {

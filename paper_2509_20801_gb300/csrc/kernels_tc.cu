@@ -243,7 +243,9 @@ constexpr uint32_t OZ_TMEM_COLS = 512;       // 2 buffers x 8 accumulators x 32 
 constexpr int OZ_EMPTY = -2000;              // exponent of an all-zero row or column
 // 16 warps stage and read out (TMEM lanes 32 (w % 4)): slicing and reading out
 // are some 1,500 instructions a thread and sub-tile at 8 warps, whose latency
-// two warps a scheduler do not cover (0.8 instructions a clock)
+// two warps a scheduler do not cover (0.8 instructions a clock).  Over the
+// factorization of 1024 x 512 in 4 strips the update takes 5.65 ms with 16
+// warps and 6.32 with 8, the column panel 2.05 and 2.47.
 constexpr int OZ_WORKERS = 512;
 constexpr int OZ_THREADS = OZ_WORKERS + 32;  // plus one warp that issues the MMAs
 constexpr int OZ_SINK = 4;                   // columns a thread reads out at a time

@@ -43,8 +43,8 @@
 // FP64 in column order, the association of the complex64 products.
 //
 // Measured against FP64 multiply-adds, one application: 4096 x 1024 nodes in
-// 16 strips 7.84 -> 5.41 ms, 2048 x 512 one strip after another (8 strips)
-// 10.5 -> 5.7 ms, 200 x 200 in 2 strips 475 -> 230 us (there the overlapped
+// 16 strips 7.89 -> 4.89 ms, 2048 x 512 one strip after another (8 strips)
+// 10.6 -> 5.4 ms, 200 x 200 in 2 strips 479 -> 205 us (there the overlapped
 // launches of consecutive levels count as much as the products).  What bounds
 // it now is the latency of the dependent loads ahead of a warp's products
 // (long-scoreboard stalls at 16 warps an SM), not a pipe.
