@@ -290,8 +290,9 @@ stdd_status stdd_set_profiling(stdd_ctx *ctx, int level);
 /* Execution options; none of them changes a computed value.
  *   STDD_OPT_GRAPHS   (default 1): replay captured CUDA graphs of the M^-1
  *                     application (one graph per input/output buffer pair,
- *                     captured on first use; the first use must not happen
- *                     inside the caller's own stream capture).
+ *                     captured on the second use since the factorization;
+ *                     no use may happen inside the caller's own stream
+ *                     capture).
  *   STDD_OPT_AUTOTUNE (default 1): choose the substitution launch shapes per
  *                     tree level by timing them once per level shape.
  *   STDD_OPT_LEAF     (default 16): nested-dissection leaf size in nodes

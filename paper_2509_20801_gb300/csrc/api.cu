@@ -14,6 +14,7 @@
 #include <memory>
 #include <mutex>
 #include <new>
+#include <set>
 #include <stdexcept>
 #include <string>
 #include <vector>
@@ -480,6 +481,25 @@ struct stdd_ctx {
     long long kernels;
   };
   std::map<std::vector<const void *>, GraphEntry> minv_graphs;
+  // and the lists used once since the factorization.  A list's first use goes
+  // out launch by launch: capturing and instantiating a graph costs the host
+  // more than the launches, which stay ahead of the GPU, and a solve that
+  // ends before a restart uses every pair of Krylov vectors once (factor and
+  // solve of 2048 x 512 in 8 strips one after another, four applications of
+  // some 700 launches: 66 ms when each was captured, 52 to 58 so).
+  std::set<std::vector<const void *>> minv_used;
+  template <typename F> void launch_or_replay(const std::vector<const void *> &key, F &&enqueue) {
+    auto it = minv_graphs.find(key);
+    if (it == minv_graphs.end()) {
+      if (minv_used.insert(key).second) {
+        enqueue();
+        return;
+      }
+      it = minv_graphs.emplace(key, capture(enqueue)).first;
+    }
+    CK(cudaGraphLaunch(it->second.exec, stream));
+    stdd::count_launch((int)it->second.kernels);
+  }
   // Capture the launches f() enqueues into an instantiated graph.  Any
   // exception thrown while capturing (a refused argument, a CUDA error) ends
   // the capture first, so the stream never stays in capture mode.  Kernels
@@ -513,11 +533,6 @@ struct stdd_ctx {
     return GraphEntry{ex, kernels};
   }
 
-  // captured graph of the numeric factorization, valid while every argument
-  // its launches were captured with (all levels' MfArgs bytes) is unchanged
-  cudaGraphExec_t factor_graph = nullptr;
-  long long factor_graph_kernels = 0;
-  std::vector<unsigned char> factor_graph_key;
   template <typename R> void enqueue_factor();
   bool use_graphs = true;
   // preconditioner order: 0 additive (Algorithm 1), 1 symmetric
@@ -554,9 +569,7 @@ struct stdd_ctx {
   void clear_graphs() {
     for (auto &kv : minv_graphs) cudaGraphExecDestroy(kv.second.exec);
     minv_graphs.clear();
-    if (factor_graph) cudaGraphExecDestroy(factor_graph);
-    factor_graph = nullptr;
-    factor_graph_key.clear();
+    minv_used.clear();
   }
   template <typename R> void factor_t();
   template <typename R> void tune_update_tiles();
@@ -623,7 +636,7 @@ double stdd_ctx::pivot_floor() const {
 
 MfArgs stdd_ctx::mf_args(int par, bool solve) const {
   MfArgs a;
-  std::memset(&a, 0, sizeof a);  // padding too: the bytes key the factorization graph
+  std::memset(&a, 0, sizeof a);
   a.fronts = d_fronts.as<FrontDev>();
   a.strips = d_strips.as<StripDev>();
   a.nodes = d_nodes.as<int>();
@@ -1253,37 +1266,7 @@ template <typename R> void stdd_ctx::tune_update_tiles() {
 template <typename R> void stdd_ctx::factor_t() {
   factor_prepare();
   const int span = pbegin(PH_FACTOR);
-  if (use_graphs && prof < 2) {
-    // one replayed graph for all levels (captured again whenever a pointer
-    // or value the launches were captured with has changed)
-    std::vector<unsigned char> key;
-    auto put = [&](const void *p, size_t nb) {
-      const unsigned char *c = static_cast<const unsigned char *>(p);
-      key.insert(key.end(), c, c + nb);
-    };
-    const int tc = tc_fmt();
-    const size_t rs = sizeof(R);
-    put(&tc, sizeof tc);
-    put(&rs, sizeof rs);
-    put(&depth, sizeof depth);
-    for (int par = 0; par < 2; ++par) {
-      const MfArgs a = mf_args(par, false);
-      put(&a, sizeof a);
-    }
-    for (const LevelInfo &li : levels) put(&li, sizeof li);
-    if (!factor_graph || key != factor_graph_key) {
-      if (factor_graph) cudaGraphExecDestroy(factor_graph);
-      factor_graph = nullptr;
-      const GraphEntry ge = capture([&] { enqueue_factor<R>(); });
-      factor_graph_kernels = ge.kernels;
-      factor_graph = ge.exec;
-      factor_graph_key = key;
-    }
-    CK(cudaGraphLaunch(factor_graph, stream));
-    stdd::count_launch((int)factor_graph_kernels);
-  } else {
-    enqueue_factor<R>();
-  }
+  enqueue_factor<R>();
   pend(span);
   int flag = 0;
   CK(cudaMemcpyAsync(&flag, d_flag.p, sizeof(int), cudaMemcpyDeviceToHost, stream));
@@ -1595,12 +1578,7 @@ void stdd_ctx::apply_op_band(const std::vector<const double2 *> &ss, const std::
       key.push_back(ss[i]);
       key.push_back(ys[i]);
     }
-    auto it = minv_graphs.find(key);
-    if (it == minv_graphs.end()) {
-      it = minv_graphs.emplace(key, capture([&] { enqueue_op_band(ss, ys); })).first;
-    }
-    CK(cudaGraphLaunch(it->second.exec, stream));
-    stdd::count_launch((int)it->second.kernels);
+    launch_or_replay(key, [&] { enqueue_op_band(ss, ys); });
   } else {
     enqueue_op_band(ss, ys);
   }
@@ -1640,16 +1618,10 @@ void stdd_ctx::apply_minv_multi(const std::vector<const double2 *> &vs, const st
       key.push_back(vs[i]);
       key.push_back(zs[i]);
     }
-    auto it = minv_graphs.find(key);
-    if (it == minv_graphs.end()) {
-      it = minv_graphs.emplace(key, capture([&] { enqueue_minv(vs, zs); })).first;
-    }
-    CK(cudaGraphLaunch(it->second.exec, stream));
-    stdd::count_launch((int)it->second.kernels);
-    pend(span);
-    return;
+    launch_or_replay(key, [&] { enqueue_minv(vs, zs); });
+  } else {
+    enqueue_minv(vs, zs);
   }
-  enqueue_minv(vs, zs);
   pend(span);
   CK(cudaGetLastError());
 }
