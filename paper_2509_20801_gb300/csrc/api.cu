@@ -1689,7 +1689,7 @@ void stdd_ctx::ensure_krylov(int m) {
   d_x.alloc(n * nq * sizeof(double2));
   d_r.alloc(n * sizeof(double2));
   d_w.alloc(n * sizeof(double2));
-  d_part.alloc((size_t)stdd::krylov_partial_blocks() * (m + 2) * sizeof(double2));
+  d_part.alloc((size_t)stdd::krylov_partial_pairs(m, nq) * sizeof(double2));
   d_h.alloc((size_t)(2 * (m + 2)) * nq * sizeof(double2));
   d_nrm.alloc((4 + 2 * (size_t)nq) * sizeof(double));
   d_y.alloc((size_t)(m + 1) * nq * sizeof(double2));

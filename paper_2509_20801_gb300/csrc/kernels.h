@@ -276,7 +276,8 @@ struct KrylovBatch {
   int64_t off[KRYLOV_BATCH];
 };
 // h[q ldh + i] = sum_g conj(V_i[g]) V_m[g], i < m; with self_norm, entry m is
-// (||V_m||^2, 0) as well.  partial: krylov_partial_blocks() * (m + 1) pairs.
+// (||V_m||^2, 0) as well.  partial:
+// krylov_partial_pairs(longest m, right-hand sides) pairs.
 void launch_mdot(const KrylovBatch &B, const double2 *V, int64_t ldv, int m, int64_t n, double2 *partial, double2 *h,
                  int64_t ldh, cudaStream_t st, int self_norm = 0);
 // V_m -= sum_i h[q ldh + i] V_i, nrm2[q ldn] = ||V_m||^2 (partials then a fixed-order sum)
@@ -292,7 +293,7 @@ void launch_maxpy(const double2 *Z, int64_t ldz, int m, const double2 *y, double
 void launch_norm2(const double2 *x, int64_t n, double *partial, double *nrm2, cudaStream_t st);
 // y = alpha * x (alpha real, read from device)
 void launch_scale(const double2 *x, const double *inv_norm2, double2 *y, int64_t n, cudaStream_t st);
-int krylov_partial_blocks();
+int64_t krylov_partial_pairs(int m, int bases);
 
 // ---- learned initial guess (kernels_nn.cu): FP32 NCHW activations
 // out = conv3x3(in) + bias (zero padding, optional ReLU); flip = 1 applies

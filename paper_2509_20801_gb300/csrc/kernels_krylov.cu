@@ -223,21 +223,27 @@ inline int nblocks_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<in
 
 }  // namespace
 
-int krylov_partial_blocks() { return NBLK; }
-
 namespace {
-// chunks of a basis: NBLK blocks in all over `share` (groups x bases), each
-// of at least two elements a thread
-int chunks_for(int64_t n, int64_t share) {
-  const int64_t most = std::max<int64_t>(1, NBLK / std::max<int64_t>(1, share));
+// Chunks of a basis whose vectors fall into `groups`: NBLK blocks over the
+// groups, each of at least two elements a thread.  The number of bases does
+// not enter: the chunks set the order of the sums, and a right-hand side's
+// must not depend on how many others still iterate.
+int chunks_for(int64_t n, int64_t groups) {
+  const int64_t most = std::max<int64_t>(1, NBLK / std::max<int64_t>(1, groups));
   return (int)std::max<int64_t>(1, std::min<int64_t>(most, (n + 2 * TPB - 1) / (2 * TPB)));
 }
 }  // namespace
 
+int64_t krylov_partial_pairs(int m, int bases) {
+  // chunks x (vectors + 1) of a basis: NBLK / groups chunks of 8 groups + 1
+  // values at most, or one chunk of every vector
+  return (int64_t)std::min(bases, KRYLOV_BATCH) * std::max(NBLK * (GROUP + 1), m + 2);
+}
+
 void launch_mdot(const KrylovBatch &B, const double2 *V, int64_t ldv, int m, int64_t n, double2 *partial, double2 *h,
                  int64_t ldh, cudaStream_t st, int self_norm) {
   const int groups = (m + GROUP - 1) / GROUP, mt = m + (self_norm ? 1 : 0);
-  const int nb = chunks_for(n, (int64_t)groups * B.n);
+  const int nb = chunks_for(n, groups);
   k_mdot<<<dim3(nb, groups, B.n), TPB, 0, st>>>(B, V, ldv, m, n, partial, self_norm);
   k_reduce_c<<<dim3((mt + 7) / 8, B.n), 256, 0, st>>>(B, partial, nb, mt, h, ldh);
   count_launch(2);
@@ -245,7 +251,7 @@ void launch_mdot(const KrylovBatch &B, const double2 *V, int64_t ldv, int m, int
 
 void launch_maxpy_norm(const KrylovBatch &B, double2 *V, int64_t ldv, int m, const double2 *h, int64_t ldh, int64_t n,
                        double *partial, double *nrm2, int64_t ldn, cudaStream_t st) {
-  const int nb = chunks_for(n, B.n);
+  const int nb = chunks_for(n, 1);
   k_maxpy_norm<<<dim3(nb, B.n), TPB, 0, st>>>(B, V, ldv, m, h, ldh, n, partial);
   k_reduce_r<<<B.n, 32, 0, st>>>(B, partial, nb, nrm2, ldn);
   count_launch(2);
@@ -253,7 +259,7 @@ void launch_maxpy_norm(const KrylovBatch &B, double2 *V, int64_t ldv, int m, con
 
 void launch_scale_basis(const KrylovBatch &B, double2 *V, int64_t ldv, int m, const double *nrm2, int64_t ldn,
                         int64_t n, cudaStream_t st) {
-  k_scale_basis<<<dim3(chunks_for(n, B.n), B.n), TPB, 0, st>>>(B, V, ldv, m, nrm2, ldn, n);
+  k_scale_basis<<<dim3(chunks_for(n, 1), B.n), TPB, 0, st>>>(B, V, ldv, m, nrm2, ldn, n);
   count_launch();
 }
 
