@@ -677,8 +677,8 @@ def run_ours(args, rank, world, local_rank):
                                       reorth_passes_per_step=extra, gbs=by / t / 1e9, tflops=fl / t / 1e12)
     # per-kernel rooflines from the launch-by-launch profile: the two
     # Gauss-Jordan elimination kernels (flops, ALU-bound) and the two
-    # substitution sweeps (factor bytes against HBM; complex128 products run
-    # as digit products on the tensor cores, not on the FP64 pipe)
+    # substitution sweeps (factor bytes; FP64 arithmetic is ALU-bound on this
+    # part at 0.5 flop/byte, complex64 is HBM-bound)
     alu_pk = fp64_tf if prec == S.STDD_PREC_FP64 else fp32_tf
     alu_src = "measured cuBLAS DGEMM" if prec == S.STDD_PREC_FP64 else "measured cuBLAS SGEMM"
     tensor = prec in (S.STDD_PREC_C64_BF16, S.STDD_PREC_C64_FP16)
@@ -698,7 +698,10 @@ def run_ours(args, rank, world, local_rank):
                      peak_source=peaks["source_bf16"])
         elif kind == "flops":
             k = dict(bound="alu", achieved=u / t / 1e12, peak=alu_pk, unit="TFLOP/s", peak_source=alu_src)
-        else:                            # sweeps: factor bytes
+        elif prec == S.STDD_PREC_FP64:   # sweep, complex128: 8 flops per 16-byte entry
+            k = dict(bound="alu", achieved=u / 2 / t / 1e12, peak=fp64_tf, unit="TFLOP/s",
+                     peak_source="measured cuBLAS DGEMM")
+        else:
             k = dict(bound="hbm", achieved=u / t / 1e9, peak=peaks["hbm_gbs"], unit="GB/s",
                      peak_source=peaks["source_hbm"])
         k.update(frac=k["achieved"] / k["peak"], ms_per_step=ms, launches_per_step=calls,

@@ -24,7 +24,6 @@
 #include "../../include/stdd.h"
 #include "common.cuh"
 #include "kernels.h"
-#include "mf_fixed.cuh"
 #include "symbolic.h"
 
 using stdd::FrontDev;
@@ -249,7 +248,6 @@ struct stdd_ctx {
   bool oz_active() const { return fp64_tc && sym_active() && prec == STDD_PREC_FP64; }
   DBuf d_lsx, d_lsy;
   DBuf d_sweep;     // the complex128 substitutions' front records
-  DBuf d_fexp;      // exponents of the fixed-point complex128 factors
   DBuf d_segpart;   // partial sums of the grid-split substitution products
   int forced_split = 0;   // STDD_OPT_SWEEP_SPLIT: 0 tuned, else 1, 2, 4, 8 or MF_SPLIT_GRID
   int64_t nfronts = 0, factor_entries = 0;
@@ -603,7 +601,8 @@ struct stdd_ctx {
   // automatic choice: complex64 sweeps run persistent (2 blocks per SM);
   // complex128 ones gain more from the per-level kernels' registers and
   // overlapped launches than from saving launches (2048 x 512, 8 strips one
-  // after another: 5.3 ms an application against 9.1)
+  // after another: 9.3 ms an application against 10.9 with one block an SM
+  // and 11.7 with two)
   int persistent_eff() const { return persistent >= 0 ? persistent : (prec == STDD_PREC_FP64 ? 0 : 2); }
   long long sweep_wait = 1ll << 22;   // polls of a grid-barrier wait before it gives up
   DBuf d_striplv, d_bar, d_sweep_flag;
@@ -664,9 +663,7 @@ MfArgs stdd_ctx::mf_args(int par, bool solve) const {
   a.panel = pivoting ? d_panel.p : nullptr;
   a.sym = sym_active() ? 1 : 0;
   a.segpart = d_segpart.p;
-  a.fexp = d_fexp.as<short>();
   a.sweep = d_sweep.as<stdd::SweepFront>();
-  a.fx_scale = std::max(-200, std::min(200, (int)std::ilogb(2.0 / (dx * dx) + 2.0 / (dy * dy))));
   a.fp64_tc = oz_active() ? 1 : 0;
   a.lsx = a.sym ? d_lsx.as<double2>() : nullptr;
   a.lsy = a.sym ? d_lsy.as<double2>() : nullptr;
@@ -887,7 +884,7 @@ void stdd_ctx::build_structure() {
   lvl_up.assign(depth, std::vector<int>(nsub + 1, 0));
   lvl_down.assign(depth, std::vector<int>(nsub + 1, 0));
   int64_t ws_need[2] = {0, 0};
-  int64_t piv_run = 0, exp_run = 0;
+  int64_t piv_run = 0;
   panel_need = 0;
   ub_elems[0] = ub_elems[1] = 0;
   for (int L = 0; L < depth; ++L) {
@@ -919,9 +916,7 @@ void stdd_ctx::build_structure() {
         d.u_off = u_run;
         d.piv_off = piv_run;
         d.pan_off = pan_run;
-        d.exp_off = exp_run;
         piv_run += sf.p;
-        exp_run += stdd::fx_exps(sf.p, sf.b);
         if (sf.p + sf.b > stdd::MF_SMALL) pan_run += (int64_t)sf.p * stdd::MF_NB;
         s_run += (int64_t)sf.b * sf.b;
         u_run += sf.b;
@@ -1067,17 +1062,14 @@ void stdd_ctx::build_structure() {
   const size_t E = elem();
   d_fac.alloc(std::max<int64_t>(1, factor_entries) * E);
   if (prec == STDD_PREC_FP64) {
-    d_fexp.alloc((size_t)std::max<int64_t>(1, exp_run) * sizeof(short));
     std::vector<stdd::SweepFront> sw(fr.size());
     for (size_t f = 0; f < fr.size(); ++f) {
       const FrontDev &d = fr[f];
       const StripDev &s = sdev[d.strip];
-      stdd::SweepFront &w = sw[f];
+      stdd::SweepFront &w = sw[f] = stdd::SweepFront{};
       const int n = d.p + d.b;
       w.down = d.fac_off;
       w.up = d.fac_off + (int64_t)d.p * n;
-      w.edown = d.exp_off;
-      w.eup = d.exp_off + stdd::fx_exps_down(d.p, d.b);
       w.nodes = d.node_off;
       w.piv = d.piv_off;
       w.voff = s.vec_off;
@@ -1087,7 +1079,6 @@ void stdd_ctx::build_structure() {
       w.Hl = s.y1 - s.y0;
       w.coef = (int)s.coef_off;
       w.ycoef = (int)s.ycoef_off;
-      w.pad = 0;
       for (int ci = 0; ci < 2; ++ci) {
         const bool has = d.child[ci] >= 0;
         w.inv[ci] = has ? d.inv_off[ci] : 0;
@@ -2064,7 +2055,7 @@ int64_t stdd_ctx::device_bytes() const {
                        &d_inv, &d_lcxm, &d_lcxp, &d_colstrip, &d_lcym, &d_lcyp, &d_rowbox, &d_fac, &d_ws[0], &d_ws[1], &d_ub[0],
                        &d_ub[1], &d_tloc, &d_wloc, &d_items, &d_flag, &d_minpiv, &d_b, &d_x, &d_r, &d_V, &d_Z, &d_w,
                        &d_part, &d_h, &d_nrm, &d_y, &d_pre, &d_fpart, &d_guess, &d_gscr, &d_pcol, &d_panel,
-                       &d_striplv, &d_bar, &d_sweep_flag, &d_lsx, &d_lsy, &d_segpart, &d_fexp, &d_sweep};
+                       &d_striplv, &d_bar, &d_sweep_flag, &d_lsx, &d_lsy, &d_segpart, &d_sweep};
   int64_t s = 0;
   for (auto *d : all) s += (int64_t)d->bytes;
   return s;

@@ -169,7 +169,6 @@ struct FrontDev {
   int64_t s_off;       // offset of F22 (b x b, col-major) in the level-parity workspace
   int64_t u_off;       // update vector (b x nrhs) at u_off * nrhs in the solve parity buffer
   int64_t piv_off;     // front-restricted pivoting: the front's p-entry column -> pivot map in MfArgs::pcol
-  int64_t exp_off;     // complex128: the rows' fixed-point exponents (mf_fixed.cuh) in MfArgs::fexp
   int64_t pan_off;     // and its pivot-panel scratch (p x MF_NB complex, per level) in MfArgs::panel
 };
 
@@ -179,11 +178,10 @@ struct FrontDev {
 // made it one longer).
 struct alignas(16) SweepFront {
   int64_t down, up;      // factor blocks [Finv H12] and -G21, in entries
-  int64_t edown, eup;    // their exponents
   int64_t nodes, piv;    // node list, column -> pivot map
   int64_t voff, u;       // the strip's local field, the front's update vector (times nrhs)
   int64_t inv[2], uc[2]; // children: extend-add maps, update vectors (uc < 0: no child)
-  int p, b, Hl, coef, ycoef, bc[2], pad;
+  int p, b, Hl, coef, ycoef, bc[2], pad[5];
 };
 
 }  // namespace stdd

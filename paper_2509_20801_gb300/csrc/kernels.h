@@ -19,17 +19,15 @@ constexpr int MF_SPLIT_GRID = 16;     // split value: one warp per (item, sub-se
 constexpr int MF_SUB = 32;            // columns per chain inside a segment (segment = chains added in order)
 static_assert(MF_SEG % MF_SUB == 0, "segments are whole sub-segments");
 constexpr int MF_PART_BYTES = 32 << 10;   // shared memory of a block's split items' chain sums
-// chains an item may have when `split` row groups (complex64: `rows` lanes)
-// or warps (complex128) of a 256-thread block share its columns, for nr
-// right-hand sides at a time; value: bytes of a complex number
-constexpr int mf_block_items(int value, int rows) { return value == 16 ? 8 : 256 / rows; }
+// chains an item may have when `split` row groups (`rows` lanes each) of a
+// 256-thread block share its columns, for nr right-hand sides at a time;
+// value: bytes of a complex number
 constexpr __host__ __device__ int mf_max_chains(int value, int rows, int split, int nr) {
-  const int items = (value == 16 ? 8 : 256 / rows) / split;
-  // a complex128 warp's lanes hold two components of 16 rows, or of 32 in two rounds
+  const int items = 256 / rows / split;
   return MF_PART_BYTES / (items * nr * rows * value);
 }
 inline bool mf_split_fits(size_t value, int rows, int split, int cols, int nr = 1) {
-  return split <= 1 || (split <= mf_block_items((int)value, rows) &&
+  return split <= 1 || (split <= 256 / rows &&
                         (cols + MF_SUB - 1) / MF_SUB <= mf_max_chains((int)value, rows, split, nr));
 }
 
@@ -74,9 +72,7 @@ struct MfArgs {
   // one partial sum per (work item, column segment, row), summed in segment
   // order by a second launch
   void *segpart;
-  short *fexp;                // complex128: exponents of the fixed-point factors
   const SweepFront *sweep;    // complex128: one record per front
-  int fx_scale;               // and the power of two Finv's columns are scaled by
 };
 
 struct LevelInfo {

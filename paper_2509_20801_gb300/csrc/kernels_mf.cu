@@ -44,7 +44,6 @@
 
 #include "common.cuh"
 #include "kernels.h"
-#include "mf_fixed.cuh"
 
 namespace stdd {
 
@@ -445,37 +444,9 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
     const int hi = max(r, c) - p, lo = min(r, c) - p;
     return cneg(cmul(ac[hi], Hm[lo * p + kc[hi]]));
   };
-  if constexpr (sizeof(R) == 8) {
-    // S as it is, the factor blocks straight to fixed point (mf_fixed.cuh),
-    // a thread per row and chain: no second pass over the small fronts
-    const int b = f.b, nd = (n + FX_COLS - 1) / FX_COLS, nu = (p + FX_COLS - 1) / FX_COLS;
-    for (int idx = t; idx < b * b; idx += TPF) {
-      const int c = idx / b, r = idx - c * b;
-      st_elem<C>(a, f, p + r, p + c, entry(p + r, p + c));
-    }
-    for (int idx = t; idx < p * nd + b * nu; idx += TPF) {
-      const bool down = idx < p * nd;
-      const int rows = down ? p : b, u = down ? idx : idx - p * nd, k = u / rows, r = u - k * rows;
-      const int c0 = k * FX_COLS, c1 = min(down ? n : p, c0 + FX_COLS), scaled = down ? p : 0;
-      int e = FX_EMPTY;
-      for (int c = c0; c < c1; ++c) {
-        const C v = entry(down ? r : p + r, c);
-        const int sh = c < scaled ? a.fx_scale : 0;
-        e = max(e, max(fx_exp(v.x, sh), fx_exp(v.y, sh)));
-      }
-      a.fexp[f.exp_off + (down ? 0 : (int64_t)p * nd) + (int64_t)k * rows + r] = (short)e;
-      ulonglong2 *W = reinterpret_cast<ulonglong2 *>(a.fac) + f.fac_off + (down ? 0 : (int64_t)p * n) + r;
-      for (int c = c0; c < c1; ++c) {
-        const C v = entry(down ? r : p + r, c);
-        const int ec = e - (c < scaled ? a.fx_scale : 0);
-        W[(int64_t)c * rows] = make_ulonglong2(fx_matrix_word(v.x, ec), fx_matrix_word(v.y, ec));
-      }
-    }
-  } else {
-    for (int idx = t; idx < n * n; idx += TPF) {
-      const int c = idx / n, r = idx - c * n;
-      st_elem<C>(a, f, r, c, entry(r, c));
-    }
+  for (int idx = t; idx < n * n; idx += TPF) {
+    const int c = idx / n, r = idx - c * n;
+    st_elem<C>(a, f, r, c, entry(r, c));
   }
   if (piv)
     for (int j = t; j < p; j += TPF) a.pcol[f.piv_off + j] = perm[j];
@@ -1000,16 +971,18 @@ __global__ void __launch_bounds__(256) mf_gj_update(MfArgs a, int f0, int k) {
 // ------------------------------------------------------- substitutions
 // Work items are (front, chunk of ROWS rows).  ROWS lanes ("row group") own
 // the ROWS rows of an item, lane = row; a 256-thread CTA holds 256/ROWS row
-// groups.  Columns are summed in fixed segments of MF_SEG columns: each
-// segment's sum starts from zero and the segment sums are added in column
-// order, so the result does not depend on how many row groups share an item
-// (split) -- split only decides which group computes which segments.  With
-// split > 1 the segment sums meet in shared memory and the first group of
-// the item adds them.  complex64: column values are gathered ROWS at a time
-// (one per lane) and broadcast by shuffles, and each lane keeps a chunk's
-// matrix loads in flight.  complex128: digit products of whole chains on the
-// tensor cores (mf_fixed.cuh), a warp per (front, chunk of ROWS rows, run of
-// chains) at both chunk heights.
+// groups.  Columns are summed in chains of MF_SUB, each from zero in column
+// order; four chains add up to a segment and the segments to the total, in
+// column order, so the result does not depend on how many row groups share
+// an item (split) -- split only decides which group sums which chains.  With
+// split > 1 the chain sums meet in shared memory and the first group of the
+// item folds them.  complex64: column values are gathered ROWS at a time (one
+// per lane) and broadcast by shuffles, and each lane keeps a chunk's matrix
+// loads in flight.  complex128: four multiply-adds an entry on a pipe that
+// takes a warp's in 64 clocks a scheduler, which sets the pace wherever loads
+// and launches are out of the way: matrix loads run ahead of the products
+// and of the previous launch's end, and vector values come from shared
+// memory.
 template <int W, typename C> __device__ __forceinline__ C shfl_w(unsigned mask, C v, int src) {
   v.x = __shfl_sync(mask, v.x, src, W);
   v.y = __shfl_sync(mask, v.y, src, W);
@@ -1080,99 +1053,70 @@ __device__ __forceinline__ void row_chains(const C *__restrict__ M, int64_t ld, 
   }
 }
 
-// Chains [k0, k1) of a complex128 front's block through the fixed-point
-// products (mf_fixed.cuh): one warp, MT x 16 rows from r0, the walk f started
-// at chain k0 and ending with chain k1 - 1.  gather(column, q) is the vector value, expo(column) the power
-// of two its column was scaled by; sink(chain, sums) receives each chain's
-// sums, sums[q][t] the lane's component (lane % 2) of its row (fx_row) of tile t.
-template <int MT, int NR, typename Gather, typename Expo, typename Sink>
-__device__ __forceinline__ void fx_chains(FxRows<MT, NR> &f, int r0, int k0, int k1, int lane, const FxLane &fl,
-                                          ulonglong2 (*xs)[FX_COLS], Gather gather, Expo expo, Sink sink) {
-  const int cend = f.cend;
-  double2 vn[NR];
-  const int cf = k0 * FX_COLS + lane;
-#pragma unroll
-  for (int q = 0; q < NR; ++q) vn[q] = cf < cend ? gather(cf, q) : czero<double2>();
-  for (int k = k0; k < k1; ++k) {
-    const int c0 = k * FX_COLS, col = c0 + lane;
-    const int sh = expo(col);
-    int ex[NR];
-    __syncwarp();      // the previous chain's products have read xs
-#pragma unroll
-    for (int q = 0; q < NR; ++q) {
-      ex[q] = __reduce_max_sync(0xffffffffu, max(fx_exp(vn[q].x, -sh), fx_exp(vn[q].y, -sh)));
-      xs[q][lane] = make_ulonglong2(fx_vector_word(vn[q].x, ex[q] + sh), fx_vector_word(vn[q].y, ex[q] + sh));
-    }
-    __syncwarp();
-    // the next chain's vector values are requested before this one's products
-    const int cn = col + FX_COLS;
-#pragma unroll
-    for (int q = 0; q < NR; ++q) vn[q] = cn < cend ? gather(cn, q) : czero<double2>();
-    double s[NR][MT];
-    if (f.rows > 0) {
-      fx_chain<MT, NR>(f, r0, c0, lane, fl, xs, ex, s);
-    } else {
-#pragma unroll
-      for (int q = 0; q < NR; ++q)
-#pragma unroll
-        for (int t = 0; t < MT; ++t) s[q][t] = 0.0;
-    }
-    sink(k, s);
-  }
-}
-// row of a 16-row tile whose sum a lane of fx_chain holds
-__device__ __forceinline__ int fx_row(int lane) { return 8 * ((lane >> 1) & 1) + (lane >> 2); }
+// The same for complex128.  A row group's matrix loads run AHEAD columns in
+// front of its products, across chains and before the first vector value has
+// arrived; vector values are staged in shared memory, ROWS columns at a time.
+// One application, with overlapped launches and the fronts' records, against
+// blocks of eight columns that one launch after another loads and broadcasts
+// by shuffles: 4096 x 1024 nodes in 16 strips 7.85 -> 7.11 ms, 2048 x 512 one
+// strip after another 10.49 -> 9.36 ms, 874 x 509 1.36 -> 1.25 ms, 200 x 200
+// 398 -> 349 us.  (Products of 8-bit digits on the tensor cores take 60 % of
+// that, but err relative to a chain's largest entry and value: the field
+// inside a metal was wrong in its third digit where these hold 1e-14.)
+template <int ROWS, int NR> struct RowWalk {
+  static constexpr int AHEAD = 8 / NR;   // (two right-hand sides: their sums take the registers)
+  const double2 *row;
+  int64_t ld;
+  int rows, cend;        // rows of the block, last column + 1 of the walk
+  double2 m[AHEAD];
 
-// Factor blocks of a level's eliminated large fronts to fixed point, in place: one
-// warp per 32 rows of a chain, lane = row, 32 columns in registers.  Reads
-// and writes every entry once (a pass at HBM speed; the preconditioner's
-// products then never convert).
-__global__ void __launch_bounds__(128) mf_to_fixed(MfArgs a, int f0, int nf, int upf) {
-  const int64_t w = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  const int fi = (int)(w / upf);
-  int u = (int)(w - (int64_t)fi * upf);
-  if (fi >= nf) return;
-  const FrontDev f = a.fronts[f0 + fi];
-  const int p = f.p, b = f.b, n = p + b;
-  if (n <= MF_SMALL) return;       // mf_gj_small wrote them so
-  const int nd = (n + FX_COLS - 1) / FX_COLS, nu = (p + FX_COLS - 1) / FX_COLS;
-  const int rd = (p + 31) / 32, ru = (b + 31) / 32;
-  int rows = p, cols = n;
-  int64_t base = f.fac_off, eo = f.exp_off;
-  const bool down = u < rd * nd;
-  if (!down) {
-    u -= rd * nd;
-    if (u >= ru * nu) return;
-    rows = b;
-    cols = p;
-    base += (int64_t)p * n;
-    eo += (int64_t)p * nd;
+  __device__ __forceinline__ void start(const double2 *__restrict__ M, int r, int rows_, int c0, int c1) {
+    rows = rows_;
+    ld = rows_;
+    cend = c1;
+    if (rows <= 0) return;                // a root's empty border
+    row = M + min(r, rows - 1);           // rows past the block repeat its last one: read, never used
+#pragma unroll
+    for (int u = 0; u < AHEAD; ++u)
+      if (c0 + u < c1) m[u] = row[(int64_t)(c0 + u) * ld];
   }
-  const int rc = (rows + 31) / 32, ch = u / rc, r = (u - ch * rc) * 32 + lane;
-  if (r >= rows) return;
-  const int c0 = ch * FX_COLS, nc = min(FX_COLS, cols - c0);
-  double2 *M = reinterpret_cast<double2 *>(a.fac) + base + (int64_t)c0 * rows + r;
-  double2 v[FX_COLS];
-  int e = FX_EMPTY;
-  const int scaled = down ? p : 0;      // columns of Finv carry 2^fx_scale
+};
+template <int ROWS, int NR, typename Gather, typename Sink>
+__device__ __forceinline__ void walk_chains(RowWalk<ROWS, NR> &w, int k0, int k1, int lane, unsigned mask,
+                                            double2 (*xs)[ROWS], Gather gather, Sink sink) {
+  constexpr int AHEAD = RowWalk<ROWS, NR>::AHEAD;
+  const int c0 = k0 * MF_SUB, c1 = w.cend;
+  double2 sub[NR], vn[NR];
 #pragma unroll
-  for (int k = 0; k < FX_COLS; ++k)
-    if (k < nc) v[k] = M[(int64_t)k * rows];
+  for (int q = 0; q < NR; ++q) {
+    sub[q] = czero<double2>();
+    vn[q] = c0 + lane < c1 ? gather(c0 + lane, q) : czero<double2>();
+  }
+  for (int cb = c0; cb < c1; cb += ROWS) {
+    __syncwarp(mask);                     // the previous columns' products have read xs
 #pragma unroll
-  for (int k = 0; k < FX_COLS; ++k)
-    if (k < nc) {
-      const int sh = c0 + k < scaled ? a.fx_scale : 0;
-      e = max(e, max(fx_exp(v[k].x, sh), fx_exp(v[k].y, sh)));
+    for (int q = 0; q < NR; ++q) xs[q][lane] = vn[q];
+    __syncwarp(mask);
+    const int cn = cb + ROWS + lane;      // the next columns' vector values are requested before these products
+#pragma unroll
+    for (int q = 0; q < NR; ++q) vn[q] = cn < c1 ? gather(cn, q) : czero<double2>();
+    if (w.rows > 0) {
+      const int nc = min(ROWS, c1 - cb);
+      for (int b = 0; b < nc; b += AHEAD)
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u)
+          if (b + u < nc) {
+#pragma unroll
+            for (int q = 0; q < NR; ++q) sub[q] = cfma(w.m[u], xs[q][b + u], sub[q]);
+            if (cb + b + u + AHEAD < c1) w.m[u] = w.row[(int64_t)(cb + b + u + AHEAD) * w.ld];
+          }
     }
-  a.fexp[eo + (int64_t)ch * rows + r] = (short)e;
+    if ((cb + ROWS) % MF_SUB == 0 || cb + ROWS >= c1) {
+      sink(cb / MF_SUB, sub);
 #pragma unroll
-  for (int k = 0; k < FX_COLS; ++k)
-    if (k < nc) {
-      const int ek = e - (c0 + k < scaled ? a.fx_scale : 0);
-      reinterpret_cast<ulonglong2 *>(M)[(int64_t)k * rows] =
-          make_ulonglong2(fx_matrix_word(v[k].x, ek), fx_matrix_word(v[k].y, ek));
+      for (int q = 0; q < NR; ++q) sub[q] = czero<double2>();
     }
+  }
 }
 
 // Going up, part 1: one warp per front forms w = [t at the pivots; 0] plus
@@ -1244,20 +1188,6 @@ __device__ __forceinline__ C wsrc_children(const WSrc<C> &s, int k, int q, C w) 
     }
   return w;
 }
-// the children's update vectors at position k, component comp alone: one
-// addition where both children have the position, none otherwise
-__device__ __forceinline__ double wsrc_children_part(const WSrc<double2> &s, int k, int q, int comp) {
-  double v[2] = {0.0, 0.0};
-  bool has[2] = {false, false};
-#pragma unroll
-  for (int ci = 0; ci < 2; ++ci)
-    if (s.uc[ci]) {
-      const int t = s.inv[ci][k];
-      has[ci] = t >= 0;
-      if (has[ci]) v[ci] = reinterpret_cast<const double *>(s.uc[ci] + (int64_t)q * s.bc[ci] + t)[comp];
-    }
-  return has[0] && has[1] ? v[0] + v[1] : has[1] ? v[1] : v[0];
-}
 // pivot position k < p; *gi = its slot in tloc / wloc
 template <typename C>
 __device__ __forceinline__ C wsrc_pivot(const MfArgs &a, const WSrc<C> &s, int k, int q, int64_t ldt, int64_t *gi) {
@@ -1307,7 +1237,7 @@ __global__ void __launch_bounds__(256) mf_up_gather(MfArgs a, int f0, int nf, in
 
 // Going up, part 2: lane = border row r;
 // u[r] = w_b[r] + sum_j (-G21)(r, j) w_p[j]  (w_b already in u).
-// NR right-hand sides share every matrix load (NR > 1 requires split == 1).
+// NR right-hand sides share every matrix load.
 // one (virtual) block of the upward products: the items of block vb
 // FUSED: no gather pass before -- the products form the gathered entries
 // themselves (WSrc, the gather's own arithmetic), the front's first row
@@ -1471,151 +1401,119 @@ __device__ __forceinline__ void down_block(const MfArgs &a, const int2 *__restri
   }
 }
 
-// The same two blocks for complex128 fronts, whose factors are fixed-point
-// numbers: one warp per work item (MT x 16 rows) or per share of its chains.
-// Chain sums are folded as in complex64: four to a segment sum, the segment
-// sums added in column order, so the split changes no result.  With split > 1
-// the chain sums meet in `part`, which holds MF_MAXCHAIN chains of 32 rows.
-// `total` of each row plus its segment sums, chain by chain in column order
-template <int MT, int NR> struct FxFold {
-  double total[NR][MT], seg[NR][MT];
-  __device__ __forceinline__ void clear() {
-#pragma unroll
-    for (int q = 0; q < NR; ++q)
-#pragma unroll
-      for (int t = 0; t < MT; ++t) total[q][t] = seg[q][t] = 0.0;
-  }
-  __device__ __forceinline__ void add(int q, int t, int k, int nk, double s) {
-    constexpr int PER = MF_SEG / FX_COLS;
-    seg[q][t] = k % PER == 0 ? s : seg[q][t] + s;
-    if (k % PER == PER - 1 || k == nk - 1) total[q][t] = k < PER ? seg[q][t] : total[q][t] + seg[q][t];
-  }
-};
+// The same two blocks for complex128, each row group with its front's record
+// in shared memory and its matrix loads ahead of level_wait.
 
-// A warp's copy of its front's record in shared memory: read once, in one
-// coalesced request, and from there where a field is needed -- the fused
-// upward products otherwise hold some thirty registers of it.
-__device__ __forceinline__ void warp_record(const MfArgs &a, int front, SweepFront *rec, int lane) {
+// A row group's copy of its front's record: read once, in one coalesced
+// request, and from there where a field is needed -- the fused upward
+// products otherwise hold some thirty registers of it.
+template <int ROWS>
+__device__ __forceinline__ void group_record(const MfArgs &a, int front, SweepFront *rec, int lane, unsigned mask) {
   static_assert(sizeof(SweepFront) == 128, "eight lanes of sixteen bytes");
-  __syncwarp();
+  __syncwarp(mask);
   if (lane < 8) reinterpret_cast<uint4 *>(rec)[lane] = reinterpret_cast<const uint4 *>(a.sweep + front)[lane];
-  __syncwarp();
+  __syncwarp(mask);
 }
 
-template <int MT, int NR, bool FUSED, bool PDL>
-__device__ __forceinline__ void up_block_fx(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
-                                            int nrhs, int64_t ldt, int vb, double *part,
-                                            ulonglong2 (*xs)[FX_COLS], SweepFront *rec) {
-  const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ipc = 8 / split, il = g / split, sidx = g - il * split;
+template <int ROWS, int NR, bool FUSED, bool PDL>
+__device__ __forceinline__ void up_block_z(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
+                                           int nrhs, int64_t ldt, int vb, double2 *part, double2 (*xs)[ROWS],
+                                           SweepFront *rec) {
+  constexpr int GROUPS = 256 / ROWS;
+  const int g = threadIdx.x / ROWS, lane = threadIdx.x % ROWS;
+  const int ipc = GROUPS / split, il = g / split, sidx = g - il * split;
   const int it = vb * ipc + il;
   const bool active = it < nitems;
-  const FxLane fl(lane);
-  int p = 0, b = 0, r0 = 0, k0 = 0, k1 = 0, nk = 0;
+  const unsigned mask = ROWS == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
+  int p = 0, b = 0, y = 0, k0 = 0, k1 = 0, nk = 0;
   if (active) {
     const int2 item = items[it];
-    warp_record(a, item.x, rec, lane);
+    group_record<ROWS>(a, item.x, rec, lane, mask);
     p = rec->p;
     b = rec->b;
-    r0 = item.y * 16 * MT;
-    nk = (p + FX_COLS - 1) / FX_COLS;
+    y = item.y;
+    nk = (p + MF_SUB - 1) / MF_SUB;
     k0 = sidx * nk / split;
     k1 = (sidx + 1) * nk / split;
   }
-  double2 *wl = reinterpret_cast<double2 *>(a.wloc);
-  double *mine = part + (int64_t)il * mf_max_chains(16, 16 * MT, split, NR) * NR * MT * 32 + lane;
+  const int r = y * ROWS + lane;
+  double2 *wl = reinterpret_cast<double2 *>(a.wloc), *u = reinterpret_cast<double2 *>(a.ub_cur);
+  double2 *mine = part + (int64_t)il * mf_max_chains(16, ROWS, split, NR) * NR * ROWS + lane;
   for (int q0 = blockIdx.y * NR; q0 < nrhs; q0 += gridDim.y * NR) {
-    FxRows<MT, NR> f;
+    RowWalk<ROWS, NR> w;
     if (active)   // -G21, b x p, ld b
-      f.start(reinterpret_cast<const double2 *>(a.fac) + rec->up, a.fexp + rec->eup, r0, b, k0 * FX_COLS,
-              min(p, k1 * FX_COLS), lane);
+      w.start(reinterpret_cast<const double2 *>(a.fac) + rec->up, r, b, k0 * MF_SUB, min(p, k1 * MF_SUB));
     if (PDL) level_wait();
-    double w0[NR][MT];     // the children's update vectors at the item's rows
+    ChainFold<double2, NR> fold;
 #pragma unroll
-    for (int q = 0; q < NR; ++q)
-#pragma unroll
-      for (int t = 0; t < MT; ++t) {
-        const int r = r0 + 16 * t + fx_row(lane);
-        const int64_t at = (int64_t)(q0 + q) * b + r;
-        w0[q][t] = 0.0;
-        if (sidx == 0 && r < b && q0 + q < nrhs)
-          w0[q][t] = FUSED ? wsrc_children_part(wsrc_make(a, *rec, nrhs), p + r, q0 + q, lane & 1)
-                           : reinterpret_cast<const double *>(a.ub_cur)[2 * (rec->u * nrhs + at) + (lane & 1)];
-      }
-    FxFold<MT, NR> fold;
-    fold.clear();
+    for (int q = 0; q < NR; ++q) {
+      fold.total[q] = fold.seg[q] = czero<double2>();
+      if (sidx == 0 && r < b && q0 + q < nrhs)
+        fold.total[q] = FUSED ? wsrc_children(wsrc_make(a, *rec, nrhs), p + r, q0 + q, czero<double2>())
+                              : u[rec->u * nrhs + (int64_t)(q0 + q) * b + r];
+    }
     if (k0 < k1) {
       auto gather = [&](int j, int q) {
         if (q0 + q >= nrhs) return czero<double2>();
         const int k = a.pcol ? a.pcol[rec->piv + j] : j;
         if (!FUSED) return wl[(q0 + q) * ldt + rec->voff + a.nodes[rec->nodes + k]];
         int64_t gi;
-        const double2 w = wsrc_pivot(a, wsrc_make(a, *rec, nrhs), k, q0 + q, ldt, &gi);
-        if (r0 == 0) wl[gi] = w;      // the front's first rows store w_p for the way down
-        return w;
+        const double2 v = wsrc_pivot(a, wsrc_make(a, *rec, nrhs), k, q0 + q, ldt, &gi);
+        if (y == 0) wl[gi] = v;      // the front's first rows store w_p for the way down
+        return v;
       };
-      fx_chains<MT, NR>(f, r0, k0, k1, lane, fl, xs, gather, [](int) { return 0; },
-                        [&](int k, const double(&s)[NR][MT]) {
+      walk_chains<ROWS, NR>(w, k0, k1, lane, mask, xs, gather, [&](int k, const double2(&s)[NR]) {
 #pragma unroll
-                          for (int t = 0; t < MT; ++t)
-#pragma unroll
-                            for (int q = 0; q < NR; ++q)
-                              if (split == 1) fold.add(q, t, k, nk, s[q][t]);
-                              else mine[((k * NR + q) * MT + t) * 32] = s[q][t];
-                        });
+        for (int q = 0; q < NR; ++q)
+          if (split == 1) fold.add(q, k, nk, s[q]);
+          else mine[(k * NR + q) * ROWS] = s[q];
+      });
     }
     if (split > 1) __syncthreads();
-    if (active && sidx == 0) {
+    if (active && sidx == 0 && r < b) {
 #pragma unroll
-      for (int t = 0; t < MT; ++t) {
-        const int r = r0 + 16 * t + fx_row(lane);
+      for (int q = 0; q < NR; ++q) {
         if (split > 1)
-          for (int k = 0; k < nk; ++k)
-#pragma unroll
-            for (int q = 0; q < NR; ++q) fold.add(q, t, k, nk, mine[((k * NR + q) * MT + t) * 32]);
-        if (r < b)
-#pragma unroll
-          for (int q = 0; q < NR; ++q)
-            if (q0 + q < nrhs)
-              reinterpret_cast<double *>(a.ub_cur)[2 * (rec->u * nrhs + (int64_t)(q0 + q) * b + r) + (lane & 1)] =
-                  w0[q][t] + fold.total[q][t];
+          for (int k = 0; k < nk; ++k) fold.add(q, k, nk, mine[(k * NR + q) * ROWS]);
+        if (q0 + q < nrhs) u[rec->u * nrhs + (int64_t)(q0 + q) * b + r] = fold.total[q];
       }
     }
     if (split > 1) __syncthreads();
   }
 }
 
-template <int MT, int NR, bool PDL>
-__device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
-                                              int nrhs, int64_t ldt, int vb, double *part,
-                                              ulonglong2 (*xs)[FX_COLS], SweepFront *rec) {
-  const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ipc = 8 / split, il = g / split, sidx = g - il * split;
+template <int ROWS, int NR, bool PDL>
+__device__ __forceinline__ void down_block_z(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
+                                             int nrhs, int64_t ldt, int vb, double2 *part, double2 (*xs)[ROWS],
+                                             SweepFront *rec) {
+  constexpr int GROUPS = 256 / ROWS;
+  const int g = threadIdx.x / ROWS, lane = threadIdx.x % ROWS;
+  const int ipc = GROUPS / split, il = g / split, sidx = g - il * split;
   const int it = vb * ipc + il;
   const bool active = it < nitems;
-  const FxLane fl(lane);
-  int p = 0, n = 0, r0 = 0, k0 = 0, k1 = 0, nk = 0;
+  const unsigned mask = ROWS == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
+  int p = 0, n = 0, r = 0, k0 = 0, k1 = 0, nk = 0;
   if (active) {
     const int2 item = items[it];
-    warp_record(a, item.x, rec, lane);
+    group_record<ROWS>(a, item.x, rec, lane, mask);
     p = rec->p;
     n = p + rec->b;
-    r0 = item.y * 16 * MT;
-    nk = (n + FX_COLS - 1) / FX_COLS;
+    r = item.y * ROWS + lane;
+    nk = (n + MF_SUB - 1) / MF_SUB;
     k0 = sidx * nk / split;
     k1 = (sidx + 1) * nk / split;
   }
   double2 *tv = reinterpret_cast<double2 *>(a.tloc);
   const double2 *wl = reinterpret_cast<const double2 *>(a.wloc);
-  double *mine = part + (int64_t)il * mf_max_chains(16, 16 * MT, split, NR) * NR * MT * 32 + lane;
+  double2 *mine = part + (int64_t)il * mf_max_chains(16, ROWS, split, NR) * NR * ROWS + lane;
   for (int q0 = blockIdx.y * NR; q0 < nrhs; q0 += gridDim.y * NR) {
-    FxRows<MT, NR> f;
+    RowWalk<ROWS, NR> w;
     if (active)   // p x n, ld p
-      f.start(reinterpret_cast<const double2 *>(a.fac) + rec->down, a.fexp + rec->edown, r0, p, k0 * FX_COLS,
-              min(n, k1 * FX_COLS), lane);
+      w.start(reinterpret_cast<const double2 *>(a.fac) + rec->down, r, p, k0 * MF_SUB, min(n, k1 * MF_SUB));
     if (PDL) level_wait();
-    FxFold<MT, NR> fold;
-    fold.clear();
+    ChainFold<double2, NR> fold;
+#pragma unroll
+    for (int q = 0; q < NR; ++q) fold.total[q] = fold.seg[q] = czero<double2>();
     if (k0 < k1) {
       auto gather = [&](int c, int q) {
         if (q0 + q >= nrhs) return czero<double2>();
@@ -1623,56 +1521,40 @@ __device__ __forceinline__ void down_block_fx(const MfArgs &a, const int2 *__res
         const int k = c < p && a.pcol ? a.pcol[rec->piv + c] : c, node = a.nodes[rec->nodes + k];
         return c < p ? wl[base + node] : cneg(tv[base + node]);
       };
-      fx_chains<MT, NR>(f, r0, k0, k1, lane, fl, xs, gather,
-                        [&](int c) { return c < p ? a.fx_scale : 0; },
-                        [&](int k, const double(&s)[NR][MT]) {
+      walk_chains<ROWS, NR>(w, k0, k1, lane, mask, xs, gather, [&](int k, const double2(&s)[NR]) {
 #pragma unroll
-                          for (int t = 0; t < MT; ++t)
-#pragma unroll
-                            for (int q = 0; q < NR; ++q)
-                              if (split == 1) fold.add(q, t, k, nk, s[q][t]);
-                              else mine[((k * NR + q) * MT + t) * 32] = s[q][t];
-                        });
+        for (int q = 0; q < NR; ++q)
+          if (split == 1) fold.add(q, k, nk, s[q]);
+          else mine[(k * NR + q) * ROWS] = s[q];
+      });
     }
     if (split > 1) __syncthreads();
-    if (active && sidx == 0) {
+    if (active && sidx == 0 && r < p) {
 #pragma unroll
-      for (int t = 0; t < MT; ++t) {
-        const int r = r0 + 16 * t + fx_row(lane);
+      for (int q = 0; q < NR; ++q) {
         if (split > 1)
-          for (int k = 0; k < nk; ++k)
-#pragma unroll
-            for (int q = 0; q < NR; ++q) fold.add(q, t, k, nk, mine[((k * NR + q) * MT + t) * 32]);
-        if (r < p)
-#pragma unroll
-          for (int q = 0; q < NR; ++q)
-            if (q0 + q < nrhs)
-              reinterpret_cast<double *>(
-                  tv)[2 * ((q0 + q) * ldt + rec->voff + a.nodes[rec->nodes + r]) + (lane & 1)] = fold.total[q][t];
+          for (int k = 0; k < nk; ++k) fold.add(q, k, nk, mine[(k * NR + q) * ROWS]);
+        if (q0 + q < nrhs) tv[(q0 + q) * ldt + rec->voff + a.nodes[rec->nodes + r]] = fold.total[q];
       }
     }
     if (split > 1) __syncthreads();
   }
 }
 
-// A work item's rows (16 or 32) go to one warp in complex128, to as many
-// lanes in complex64: items a 256-thread block holds at split 1.
-template <typename R> __host__ __device__ constexpr int block_items(int rows) {
-  return sizeof(R) == 8 ? 8 : 256 / rows;
-}
-
 // one (virtual) block of products of either precision; `part` holds the
-// segment sums of split items, the warps' vector words follow it
+// chain sums of split items; complex128: the staged vector values and the
+// records follow it (double2 units)
 template <typename R, int NR>
-constexpr int SWEEP_SMEM = MF_PART_BYTES / (2 * sizeof(R)) + (sizeof(R) == 8 ? 8 * NR * FX_COLS + 8 * (int)sizeof(SweepFront) / 16 : 0);
+constexpr int SWEEP_SMEM =
+    MF_PART_BYTES / (2 * sizeof(R)) + (sizeof(R) == 8 ? 256 * NR + 16 * (int)(sizeof(SweepFront) / sizeof(double2)) : 0);
 template <typename R, int ROWS, int NR, bool FUSED, bool PDL>
 __device__ __forceinline__ void up_any(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                        int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
   if constexpr (sizeof(R) == 8) {
-    auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_PART_BYTES / sizeof(double2)) + (threadIdx.x >> 5) * NR;
-    auto rec = reinterpret_cast<SweepFront *>(part + MF_PART_BYTES / sizeof(double2) + 8 * NR * FX_COLS) + (threadIdx.x >> 5);
-    up_block_fx<ROWS / 16, NR, FUSED, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs,
-                                        rec);
+    double2 *after = part + MF_PART_BYTES / sizeof(double2);
+    auto xs = reinterpret_cast<double2(*)[ROWS]>(after) + threadIdx.x / ROWS * NR;
+    auto rec = reinterpret_cast<SweepFront *>(after + 256 * NR) + threadIdx.x / ROWS;
+    up_block_z<ROWS, NR, FUSED, PDL>(a, items, nitems, split, nrhs, ldt, vb, part, xs, rec);
   } else {
     if (PDL) level_wait();
     up_block<R, ROWS, NR, FUSED>(a, items, nitems, split, nrhs, ldt, vb, part);
@@ -1682,10 +1564,10 @@ template <typename R, int ROWS, int NR, bool PDL>
 __device__ __forceinline__ void down_any(const MfArgs &a, const int2 *__restrict__ items, int nitems, int split,
                                          int nrhs, int64_t ldt, int vb, typename CT<R>::T *part) {
   if constexpr (sizeof(R) == 8) {
-    auto xs = reinterpret_cast<ulonglong2(*)[FX_COLS]>(part + MF_PART_BYTES / sizeof(double2)) + (threadIdx.x >> 5) * NR;
-    auto rec = reinterpret_cast<SweepFront *>(part + MF_PART_BYTES / sizeof(double2) + 8 * NR * FX_COLS) + (threadIdx.x >> 5);
-    down_block_fx<ROWS / 16, NR, PDL>(a, items, nitems, split, nrhs, ldt, vb, reinterpret_cast<double *>(part), xs,
-                                        rec);
+    double2 *after = part + MF_PART_BYTES / sizeof(double2);
+    auto xs = reinterpret_cast<double2(*)[ROWS]>(after) + threadIdx.x / ROWS * NR;
+    auto rec = reinterpret_cast<SweepFront *>(after + 256 * NR) + threadIdx.x / ROWS;
+    down_block_z<ROWS, NR, PDL>(a, items, nitems, split, nrhs, ldt, vb, part, xs, rec);
   } else {
     if (PDL) level_wait();
     down_block<R, ROWS, NR>(a, items, nitems, split, nrhs, ldt, vb, part);
@@ -1712,10 +1594,9 @@ __global__ void __launch_bounds__(256, 2) mf_down(MfArgs a, const int2 *__restri
 // Products split across the grid: one warp per (work item, MF_SUB-column
 // chain) anywhere in the grid writes the chain's sum per row, and a second
 // launch folds the chains into segment sums and the segment sums into the
-// total, in column order -- the association seg_dot and the in-block
-// split use, so the choice between them changes no result.  At the top tree
+// total, in column order -- the association of the in-block split, so the choice between them changes no result.  At the top tree
 // levels a few fronts carry a whole phase; an in-block split keeps an item on
-// one SM.
+// one SM, whose FP64 pipe then sets a complex128 phase's time.
 template <typename R, bool UP, bool FUSED>
 __global__ void __launch_bounds__(256) mf_seg_partial(MfArgs a, const int2 *__restrict__ items, int nitems,
                                                       int nsubmax, int64_t ldt) {
@@ -1752,19 +1633,13 @@ __global__ void __launch_bounds__(256) mf_seg_partial(MfArgs a, const int2 *__re
     return w;
   };
   if constexpr (sizeof(R) == 8) {
-    __shared__ ulonglong2 xs[8][1][FX_COLS];
-    const FxLane fl(lane);
-    const short *E = a.fexp + f.exp_off + (UP ? (int64_t)p * ((n + FX_COLS - 1) / FX_COLS) : 0);
-    double *out = reinterpret_cast<double *>(a.segpart) + u * 64 + 2 * fx_row(lane) + (lane & 1);
-    FxRows<2, 1> walk;
-    walk.start(M, E, item.y * 32, ld, c0, c1, lane);
+    __shared__ double2 xs[8][1][32];
+    RowWalk<32, 1> walk;
+    walk.start(M, r, ld, c0, c1);
     level_wait();
-    fx_chains<2, 1>(walk, item.y * 32, sg, sg + 1, lane, fl, xs[warp], gather,
-                    [&](int c) { return !UP && c < p ? a.fx_scale : 0; },
-                    [&](int, const double(&s)[1][2]) {
-                      out[0] = s[0][0];
-                      out[32] = s[0][1];
-                    });
+    walk_chains<32, 1>(walk, sg, sg + 1, lane, 0xffffffffu, xs[warp], gather, [&](int, const double2(&s)[1]) {
+      reinterpret_cast<double2 *>(a.segpart)[u * 32 + lane] = s[0];
+    });
   } else {
     level_wait();
     row_chains<32, 1, C>(M, ld, r, row, sg, sg + 1, cols, lane, 0xffffffffu, gather,
@@ -1790,15 +1665,13 @@ __global__ void __launch_bounds__(256) mf_seg_reduce(MfArgs a, const int2 *__res
   const int nsub = (cols + MF_SUB - 1) / MF_SUB, per = MF_SEG / MF_SUB;
   const C *P = reinterpret_cast<const C *>(a.segpart) + (int64_t)it * nsubmax * 32 + lane;
   C *u = reinterpret_cast<C *>(a.ub_cur) + f.u_off;
-  C w0 = czero<C>(), total = czero<C>();
-  if (UP) w0 = FUSED ? wsrc_children(wsrc_make<C>(a, f, 1), p + r, 0, czero<C>()) : u[r];
-  if (sizeof(R) == 4) total = w0;      // complex64 items start from it, complex128 ones add it last
+  C total = czero<C>();
+  if (UP) total = FUSED ? wsrc_children(wsrc_make<C>(a, f, 1), p + r, 0, czero<C>()) : u[r];
   for (int k0 = 0; k0 < nsub; k0 += per) {
     C seg = P[k0 * 32];
     for (int k = k0 + 1; k < min(k0 + per, nsub); ++k) seg = cadd(seg, P[k * 32]);
     total = cadd(total, seg);
   }
-  if (sizeof(R) == 8) total = cadd(w0, total);
   if (UP) u[r] = total;
   else reinterpret_cast<C *>(a.tloc)[a.strips[f.strip].vec_off + a.nodes[f.node_off + r]] = total;
 }
@@ -1851,7 +1724,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *flag, long long
 template <typename R, int ROWS>
 __device__ __forceinline__ void up_items(const MfArgs &a, const StripLevel &l, int64_t ldt,
                                          typename CT<R>::T *part) {
-  const int ipc = block_items<R>(ROWS) / l.split_up;
+  const int ipc = 256 / ROWS / l.split_up;
   const int nvb = (l.up_n + ipc - 1) / ipc;
   for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x)
     up_any<R, ROWS, 1, true, false>(a, a.items_sweep + l.up_first, l.up_n, l.split_up, 1, ldt, vb, part);
@@ -1860,7 +1733,7 @@ __device__ __forceinline__ void up_items(const MfArgs &a, const StripLevel &l, i
 template <typename R, int ROWS>
 __device__ __forceinline__ void down_items(const MfArgs &a, const StripLevel &l, int64_t ldt,
                                            typename CT<R>::T *part) {
-  const int ipc = block_items<R>(ROWS) / l.split_down;
+  const int ipc = 256 / ROWS / l.split_down;
   const int nvb = (l.down_n + ipc - 1) / ipc;
   for (int vb = blockIdx.x; vb < nvb; vb += gridDim.x)
     down_any<R, ROWS, 1, false>(a, a.items_sweep + l.down_first, l.down_n, l.split_down, 1, ldt, vb, part);
@@ -2014,13 +1887,6 @@ void mf_factor_level(const MfArgs &a, const LevelInfo &L, int level, cudaStream_
       }
     }
   }
-  if (sizeof(R) == 8 && L.max_n > MF_SMALL) {
-    // the substitutions read fixed-point factors (the parents only read S)
-    const int upf = (L.max_p + 31) / 32 * ((L.max_n + FX_COLS - 1) / FX_COLS) +
-                    (L.max_b + 31) / 32 * ((L.max_p + FX_COLS - 1) / FX_COLS);
-    mf_to_fixed<<<(unsigned)(((int64_t)L.nf * upf + 3) / 4), 128, 0, st>>>(a, L.f0, L.nf, upf);
-    count_launch();
-  }
 }
 
 template <typename R>
@@ -2055,7 +1921,7 @@ void mf_up_level(const MfArgs &a, const int2 *items, int nitems, int rows, int s
   }
   if (cols_max > 0)
     while (!mf_split_fits(2 * sizeof(R), rows, split, cols_max, nr)) split /= 2;
-  const int ipc = block_items<R>(rows) / split;
+  const int ipc = 256 / rows / split;
   const dim3 grid = rhs_grid((nitems + ipc - 1) / ipc, nrhs, nr);
 #define STDD_UP(RW, NRV)                                                                \
   do {                                                                                  \
@@ -2086,7 +1952,7 @@ void mf_down_level(const MfArgs &a, const int2 *items, int nitems, int rows, int
   }
   if (cols_max > 0)
     while (!mf_split_fits(2 * sizeof(R), rows, split, cols_max, nr)) split /= 2;
-  const int ipc = block_items<R>(rows) / split;
+  const int ipc = 256 / rows / split;
   const dim3 grid = rhs_grid((nitems + ipc - 1) / ipc, nrhs, nr);
 #define STDD_DOWN(RW, NRV) launch_overlapped(mf_down<R, RW, NRV>, grid, 256, 0, st, a, items, nitems, split, nrhs, ldt)
   if (rows == 16) {
