@@ -50,22 +50,17 @@ template <typename C> __host__ __device__ __forceinline__ C cconjmul(C a, C b) {
 template <typename C> __host__ __device__ __forceinline__ auto cabs2(C a) -> decltype(a.x) {
   return a.x * a.x + a.y * a.y;
 }
-// 1/x for a positive normal x by Newton's iteration y <- y + y (1 - x y) from
-// the hardware's approximation: two rounds square its error below 2^-53 twice
-// over (result within an ulp).  Five instructions on the FP64 pipe, which a
-// lone pivot's chain waits for and which a warp pays in full for one lane; the
-// correctly rounded __drcp_rn takes several times as many.
-__device__ __forceinline__ double drecip(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
-}
-// 1/a in complex128: conj(a) / |a|^2, one real reciprocal and three products;
-// |a|^2 over- or underflows for |a| outside about 1e-154 .. 1e154: the
-// callers flag pivots outside it (pivot_ok).
+// 1/a in complex128: conj(a) / |a|^2, one correctly rounded real reciprocal
+// and three products.  R. L. Smith's scaled form (CACM 5(8), 1962) costs two
+// more divisions, and on a part whose FP64 pipe retires one warp instruction
+// per 64 cycles per scheduler even one thread's scalar FP64 work costs what a
+// full warp's does.  |a|^2 must neither overflow nor underflow: |a| between
+// about 1e-154 and 1e154, far outside the stencil scale of these operators;
+// callers flag pivots outside it (pivot_ok).  (Newton's iteration from the
+// hardware's approximation takes a third of the instructions, but flushes the
+// reciprocal of |a|^2 above 2^1022 to zero.)
 __device__ __forceinline__ double2 crecip(double2 a) {
-  const double s = drecip(a.x * a.x + a.y * a.y);
+  const double s = __drcp_rn(a.x * a.x + a.y * a.y);
   return make_double2(a.x * s, -a.y * s);
 }
 // 1/a in complex64 by Smith's algorithm: the FP32 pipe is not the limit,
