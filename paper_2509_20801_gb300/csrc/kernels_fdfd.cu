@@ -30,13 +30,13 @@ __device__ __forceinline__ double2 apply_row(const GridDev &g, const double2 *__
 }
 
 // y = A x, or y = b - A x (RES), column by column: a thread keeps its row j
-// and walks ci columns, so the x-neighbours are the values it just had and
-// its y couplings stay in registers.  What bounds it is the FP64 pipe (1 flop
-// a byte against the machine's 0.16): 12 operations a node outside the PML,
-// where the couplings are real, against 15 when every node recomputes the sum
-// of its four couplings, and one new field value a node against three.  b may
-// be y itself (a node is read before it is written, by the same thread).
-// NORM: partial[block] = (sum |y|^2, sum |b|^2) of the block's nodes.
+// and walks ci columns, so the x-neighbours are the values it just had: one
+// new field value a node against three, and no division.  Products and sums
+// are grid_row's in its order, fourteen FP64 operations a node outside the
+// PML, where the couplings are real; a residual takes two more and its norms
+// four.  b may be y itself (a node is read before it is written, by the same
+// thread).  NORM: partial[block] = (sum |y|^2, sum |b|^2) of the block's
+// nodes.
 constexpr int COLT = 128;
 
 template <bool RES, bool NORM>
@@ -48,7 +48,6 @@ __global__ void __launch_bounds__(COLT) k_stencil_cols(GridDev g, const double2 
   if (j < g.ny) {
     const double2 ym = g.cym[j], yp = g.cyp[j], zero = make_double2(0.0, 0.0);
     const bool yreal = ym.y == 0.0 && yp.y == 0.0;
-    const double ys = ym.x + yp.x;
     const bool has_s = j > 0, has_n = j < g.ny - 1;
     int64_t idx = (int64_t)i0 * g.ny + j;
     double2 w = i0 > 0 ? x[idx - g.ny] : zero, c = x[idx];
@@ -66,27 +65,28 @@ __global__ void __launch_bounds__(COLT) k_stencil_cols(GridDev g, const double2 
         kn = g.eps[idx + g.ny];
       }
       double2 acc;
+      double2 d;
+      d.x = fma(g.k0sq, ke, -xm.x) - xp.x - ym.x - yp.x;
+      acc = make_double2(d.x * c.x, d.x * c.y);
       if (yreal && xm.y == 0.0 && xp.y == 0.0) {
-        const double sg = RES ? -1.0 : 1.0;
-        const double d = sg * (fma(g.k0sq, ke, -ys) - (xm.x + xp.x));
-        acc.x = fma(d, c.x, bv.x);
-        acc.y = fma(d, c.y, bv.y);
-        acc.x = fma(sg * xm.x, w.x, acc.x);
-        acc.y = fma(sg * xm.x, w.y, acc.y);
-        acc.x = fma(sg * xp.x, e.x, acc.x);
-        acc.y = fma(sg * xp.x, e.y, acc.y);
-        acc.x = fma(sg * ym.x, s.x, acc.x);
-        acc.y = fma(sg * ym.x, s.y, acc.y);
-        acc.x = fma(sg * yp.x, n.x, acc.x);
-        acc.y = fma(sg * yp.x, n.y, acc.y);
+        acc.x = fma(xm.x, w.x, acc.x);
+        acc.y = fma(xm.x, w.y, acc.y);
+        acc.x = fma(xp.x, e.x, acc.x);
+        acc.y = fma(xp.x, e.y, acc.y);
+        acc.x = fma(ym.x, s.x, acc.x);
+        acc.y = fma(ym.x, s.y, acc.y);
+        acc.x = fma(yp.x, n.x, acc.x);
+        acc.y = fma(yp.x, n.y, acc.y);
       } else {
-        const double2 d = make_double2(fma(g.k0sq, ke, -ys) - (xm.x + xp.x), -(xm.y + xp.y) - (ym.y + yp.y));
-        acc = cfma(xm, w, cmul(d, c));
+        d.y = -xm.y - xp.y - ym.y - yp.y;
+        acc.x = fma(d.x, c.x, -__dmul_rn(d.y, c.y));
+        acc.y = fma(d.y, c.x, acc.y);
+        acc = cfma(xm, w, acc);
         acc = cfma(xp, e, acc);
         acc = cfma(ym, s, acc);
         acc = cfma(yp, n, acc);
-        if (RES) acc = csub(bv, acc);
       }
+      if (RES) acc = csub(bv, acc);
       y[idx] = acc;
       if (NORM) {
         ny2 = fma(acc.x, acc.x, fma(acc.y, acc.y, ny2));
@@ -128,10 +128,11 @@ __global__ void __launch_bounds__(TPB) k_sum_pairs(const double2 *__restrict__ p
 }
 
 // Columns a thread walks: enough blocks for sixteen on every SM, else longer
-// walks, which read fewer columns twice.  4096 x 1024, a residual: 231 us with
-// blocks for eight, 218 with sixteen, 217 with 32, 237 with 64 (352 us with
-// one node a thread and copies into buffers of the library's own); an operator
-// on 200 x 200, one column a thread, 24.5 -> 15.5 us.
+// walks, which read fewer columns twice.  4096 x 1024, a residual waited for:
+// 261 us with blocks for eight, 247 with sixteen, 247 with 32, 262 with 64;
+// among others 239 us (348 us with one node a thread and copies into buffers
+// of the library's own).  An operator on 200 x 200, one column a thread, 24.4
+// -> 15.4 us.
 inline int stencil_cols(const GridDev &g) {
   const int64_t rows = (g.ny + COLT - 1) / COLT;
   return (int)std::max<int64_t>(1, rows * g.nx / (152 * 16));
