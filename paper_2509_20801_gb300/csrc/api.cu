@@ -484,7 +484,7 @@ struct stdd_ctx {
   // more than the launches, which stay ahead of the GPU, and a solve that
   // ends before a restart uses every pair of Krylov vectors once (factor and
   // solve of 2048 x 512 in 8 strips one after another, four applications of
-  // some 700 launches: 66 ms when each was captured, 52 to 58 so).
+  // some 700 launches: 84 to 86 ms when each was captured, 75 so).
   std::set<std::vector<const void *>> minv_used;
   template <typename F> void launch_or_replay(const std::vector<const void *> &key, F &&enqueue) {
     auto it = minv_graphs.find(key);

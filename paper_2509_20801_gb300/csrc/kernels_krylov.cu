@@ -39,11 +39,9 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
   return s;
 }
 
-// The bases of the right-hand sides that iterate: basis z is base + off[z],
-// its vectors ldv apart, the vector to be orthogonalised w + off[z].
-// GROUP values of a thread added over the warp, value q left in lane q * 32 /
-// GROUP: halving the values each round takes 2 GROUP - 1 exchanges where
-// GROUP separate sums take 5 GROUP.
+// N = 2 GROUP values of a thread added over the warp, value q left in lanes
+// 2 q and 2 q + 1: halving the values each round takes N exchanges where N
+// separate sums take 5 N.
 template <int N> __device__ __forceinline__ double warp_sums(double (&v)[N], int lane) {
   static_assert(N == 16, "sixteen values");
 #pragma unroll
@@ -67,7 +65,7 @@ template <int N> __device__ __forceinline__ double warp_sums(double (&v)[N], int
 // groups in every block, chunks of two elements a thread and a block-wide sum
 // for each component, the reductions took two thirds of the time (262,144
 // nodes, 40 vectors: 212 us; the FP64 pipe needs 76).  Eight bases of 262,144
-// nodes and some 25 vectors now take 397 us in one launch, the pipe's time.
+// nodes and some 25 vectors take 432 us in one launch, near the pipe's time.
 __global__ void __launch_bounds__(TPB) k_mdot(KrylovBatch B, const double2 *__restrict__ Vb, int64_t ldv, int m,
                                               int64_t n, double2 *__restrict__ partial, int self_norm) {
   __shared__ double sh[TPB / 32][2 * GROUP + 1];

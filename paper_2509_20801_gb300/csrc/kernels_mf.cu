@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(128) mf_gj_small(MfArgs a, int f0, int nf, int
   // H12(:, c) = Finv(:, k(c)) a_c, S = - a_r Finv(k(r), k(c)) a_c -- a third
   // of the sweep's multiply-adds at 16 pivots and 16 border nodes.  FP64-pipe
   // bound: the fronts of up to 32 rows of a 1024 x 512 grid in 4 strips took
-  // 3.04 ms when every front was swept whole, 1.97 ms so.
+  // 3.04 ms when every front was swept whole, 1.81 ms so.
   const bool leaf = sym && !has[0] && !has[1];
   const int m = leaf ? p : n;                       // rows and columns swept
   const int lds = leaf ? (p | 1) : ld;

@@ -294,7 +294,7 @@ __device__ __forceinline__ void oz_slice(double x, int er, uint32_t (&s)[OZ_S]) 
   }
 }
 
-// barrier over the 8 staging / read-out warps only (the MMA warp runs on)
+// barrier over the staging / read-out warps only (the MMA warp runs on)
 __device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(OZ_WORKERS) : "memory"); }
 
 // V 2^e as a double: one rounding of V (|V| < 2^62), then the exact power of
@@ -369,7 +369,7 @@ __device__ int oz_rows(OzSmem &sm, int kc, int ncols, CLoad cload, RLoad rload, 
   const uint32_t idesc = tcx::instr_desc_f16(1, 128, OZ_NC);
   const int drow = (warp & 3) * 32 + lane, er = drow >> 1, comp = drow & 1;
   const int hq = 8 * (warp >> 2);   // each four warps read 8 columns of a sub-tile, OZ_SINK at a time
-  // read out sub-tile s: the 8 order sums of 16 columns at a time
+  // read out sub-tile s: the 8 order sums of OZ_SINK columns at a time
   auto drain = [&](int s) {
     const int buf = s & 1;
     // one decision per warp: the reads below are warp-collective
